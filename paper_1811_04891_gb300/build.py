@@ -16,8 +16,11 @@ SRC = os.path.join(HERE, "csrc")
 OUT = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT, "libfindpts_gb.so")
 SOURCES = ["fp_host.cu", "fp_setup.cu", "fp_scan.cu", "fp_find.cu", "fp_find2.cu", "fp_eval.cu", "fp_static.cu",
-           "fp_batch.cu", "fp_flux.cu", "fp_stream.cu", "fp_probe.cu"]
-HEADERS = ["fp_common.cuh", "fp_internal.h", "fp_handle.h", "fp_rank.cuh"]
+           "fp_batch.cu", "fp_flux.cu", "fp_stream.cu", "fp_probe.cu", "fp_solve.cu", "fp_tile_mixed.cu"]
+HEADERS = ["fp_common.cuh", "fp_internal.h", "fp_handle.h", "fp_rank.cuh", "fp_newton.cuh", "fp_tile.cuh",
+           "fp_tile_launch.cuh"]
+# sources compiled once per order n, with flags of their own
+PER_ORDER = {"fp_solve.cu": (range(2, 17), []), "fp_tile_mixed.cu": ([5, 7, 8, 9, 10], ["-fmad=false"])}
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 
@@ -48,10 +51,13 @@ def build(force: bool = False, verbose: bool = False, ptxas_v: bool = False) -> 
         return LIB
     os.makedirs(OUT, exist_ok=True)
     extra = ["-Xptxas", "-v"] if ptxas_v else []
-    cmds = []
+    cmds, objs = [], []
     for f in SOURCES:
-        obj = os.path.join(OUT, f.replace(".cu", ".o"))
-        cmds.append([nvcc(), *_flags(extra), "-c", os.path.join(SRC, f), "-o", obj])
+        orders, flags = PER_ORDER.get(f, ([0], []))
+        for k in orders:
+            objs.append(os.path.join(OUT, f.replace(".cu", f"_{k}.o" if k else ".o")))
+            cmds.append([nvcc(), *_flags(extra), *flags, *([f"-DFP_N={k}"] if k else []), "-c", os.path.join(SRC, f),
+                         "-o", objs[-1]])
 
     def run(cmd):
         r = subprocess.run(cmd, capture_output=True, text=True)
@@ -64,7 +70,6 @@ def build(force: bool = False, verbose: bool = False, ptxas_v: bool = False) -> 
             sys.stderr.write(r.stdout + r.stderr)
         if r.returncode != 0:
             raise RuntimeError("nvcc failed: " + " ".join(cmd) + "\n" + r.stdout + r.stderr)
-    objs = [os.path.join(OUT, f.replace(".cu", ".o")) for f in SOURCES]
     tmp = LIB + f".{os.getpid()}.tmp"
     link = [nvcc(), *ARCH, "-shared", "-o", tmp, *objs, "-Xcompiler", "-fPIC"]
     r = subprocess.run(link, capture_output=True, text=True)

@@ -60,6 +60,7 @@ struct Group {
     double* coords = nullptr;
     float* coords32 = nullptr;
     float* coords32lo = nullptr;
+    unsigned char* digits = nullptr;   // orders of the tile kernels
     ElemBox* boxes = nullptr;
     double* dist = nullptr;
     double* fields = nullptr;
@@ -105,7 +106,7 @@ void release(T*& p)
 
 void release_group(Group& g)
 {
-    release(g.coords); release(g.coords32); release(g.coords32lo); release(g.boxes); release(g.dist);
+    release(g.coords); release(g.coords32); release(g.coords32lo); release(g.digits); release(g.boxes); release(g.dist);
     release(g.fields); release(g.fields_df); release(g.d_tab);
     if (g.st) cudaStreamDestroy(g.st);
     if (g.done) cudaEventDestroy(g.done);
@@ -232,9 +233,11 @@ struct fp_batch {
     uint32_t* smask = nullptr;
     int32_t *pair_elem = nullptr, *pair_pt = nullptr, *order = nullptr, *ecount = nullptr, *estart = nullptr;
     int32_t* fb_list = nullptr;
-    int32_t* gcount = nullptr;    // [2 * groups]: Newton work-queue counter, fallback counter
+    int32_t* pause_list = nullptr;
+    float* jst = nullptr;         // [9][cap] mixed form: Jacobians between the Newton stage's two launches
+    int32_t* gcount = nullptr;    // [3 * groups]: Newton work-queue counter, fallback counter, listed solves
     double *pres = nullptr, *prst = nullptr;
-    double2* pstate = nullptr;    // FP64 form: state of solves paused by the first Newton pass
+    double2* pstate = nullptr;    // state of solves paused by the first Newton pass
     int32_t* inv = nullptr;       // sorted position of each pair slot
     unsigned long long* band = nullptr;
     cudaEvent_t fork = nullptr, fork2 = nullptr;
@@ -259,7 +262,7 @@ static void batch_release(fp_batch* b)
     release(b->d_inst); release(b->d_p0); release(b->d_rinst); release(b->d_rgrp); release(b->he_all);
     release(b->sub_all); release(b->cnt); release(b->smask); release(b->off); release(b->scan_tmp); release(b->pair_elem);
     release(b->pair_pt); release(b->order); release(b->ecount); release(b->estart); release(b->fb_list);
-    release(b->gcount); release(b->pres); release(b->prst); release(b->pstate); release(b->inv); release(b->band);
+    release(b->gcount); release(b->pres); release(b->prst); release(b->pstate); release(b->inv); release(b->pause_list); release(b->jst); release(b->band);
     if (b->fork) cudaEventDestroy(b->fork);
     if (b->fork2) cudaEventDestroy(b->fork2);
     if (b->exec) cudaGraphExecDestroy(b->exec);
@@ -354,7 +357,10 @@ extern "C" fp_status fp_batch_create(fp_batch** out, int ninst, fp_handle* const
         g.fp.refine = handles[0]->refine;
         e = alloc(&g.coords, 3 * g.E * n3);
         if (e == cudaSuccess && b->mixed) e = alloc(&g.coords32, 3 * g.E * n3);
-        if (e == cudaSuccess && b->mixed) e = alloc(&g.coords32lo, 3 * g.E * n3);
+        const bool lo = b->mixed && !is_tile_order(g.n, true);
+        if (e == cudaSuccess && lo) e = alloc(&g.coords32lo, 3 * g.E * n3);
+        const int64_t db = tile_digits_bytes(g.n, b->mixed);
+        if (e == cudaSuccess && db > 0) e = alloc(&g.digits, g.E * db);
         if (e == cudaSuccess) e = alloc(&g.boxes, g.E);
         if (e == cudaSuccess && multi) e = alloc(&g.dist, g.E * n3);
         if (e == cudaSuccess && F > 0) e = alloc(&g.fields, (int64_t)F * g.E * n3);
@@ -371,10 +377,12 @@ extern "C" fp_status fp_batch_create(fp_batch** out, int ninst, fp_handle* const
                 if (e == cudaSuccess && b->mixed)
                     e = cudaMemcpy(g.coords32 + (a * g.E + eo) * n3, h->coords32 + a * Ei * n3,
                                    sizeof(float) * Ei * n3, cudaMemcpyDeviceToDevice);
-                if (e == cudaSuccess && b->mixed)
+                if (e == cudaSuccess && lo)
                     e = cudaMemcpy(g.coords32lo + (a * g.E + eo) * n3, h->coords32lo + a * Ei * n3,
                                    sizeof(float) * Ei * n3, cudaMemcpyDeviceToDevice);
             }
+            if (e == cudaSuccess && db > 0)
+                e = cudaMemcpy(g.digits + eo * db, h->digits, (size_t)(Ei * db), cudaMemcpyDeviceToDevice);
             if (e == cudaSuccess)
                 e = cudaMemcpy(g.boxes + eo, h->boxes, sizeof(ElemBox) * Ei, cudaMemcpyDeviceToDevice);
             if (e == cudaSuccess && g.dist) {
@@ -455,10 +463,14 @@ extern "C" fp_status fp_batch_create(fp_batch** out, int ninst, fp_handle* const
         if (e == cudaSuccess) e = alloc(&b->fb_list, b->cap);
         if (e == cudaSuccess) e = alloc(&b->ecount, b->Etot);
         if (e == cudaSuccess) e = alloc(&b->estart, b->Etot + 1);
-        if (e == cudaSuccess) e = alloc(&b->gcount, 2 * ng);
+        if (e == cudaSuccess) e = alloc(&b->gcount, 3 * ng);
         if (e == cudaSuccess) e = alloc(&b->pres, b->cap);
         if (e == cudaSuccess) e = alloc(&b->prst, 3 * b->cap);
-        if (e == cudaSuccess && !b->mixed) e = alloc(&b->pstate, b->cap);
+        bool tile = false;
+        for (auto& g : b->groups) tile = tile || is_tile_order(g.n, b->mixed);
+        if (e == cudaSuccess && (tile || !b->mixed)) e = alloc(&b->pstate, b->cap);
+        if (e == cudaSuccess && tile) e = alloc(&b->pause_list, b->cap);
+        if (e == cudaSuccess && tile && b->mixed) e = alloc(&b->jst, 9 * b->cap);
         if (e == cudaSuccess) e = alloc(&b->inv, b->cap);
         if (e == cudaSuccess) e = alloc(&b->band, 3);
         if (e == cudaSuccess) e = cudaMemset(b->band, 0, 3 * sizeof(unsigned long long));
@@ -499,6 +511,7 @@ static FindArgs group_args(const fp_batch* b, const Group& g, const double* pts)
     a.coords32 = g.coords32;
     a.coords32lo = g.coords32lo;
     a.boxes = g.boxes;
+    a.digits = g.digits;
     a.off = b->off;
     a.pair_elem = b->pair_elem;
     a.pair_pt = b->pair_pt;
@@ -510,9 +523,12 @@ static FindArgs group_args(const fp_batch* b, const Group& g, const double* pts)
     a.s_hi = b->estart + g.ebase + g.E;
     a.ebase = g.ebase;
     const int64_t gi = &g - b->groups.data();
-    a.queue = b->gcount + 2 * gi;
-    a.fb_count = b->gcount + 2 * gi + 1;
+    a.queue = b->gcount + 3 * gi;
+    a.fb_count = b->gcount + 3 * gi + 1;
+    a.pause_count = b->gcount + 3 * gi + 2;
     a.fb_list = b->fb_list;
+    a.pause_list = b->pause_list;
+    a.jst = b->jst;
     a.pstate = b->pstate;
     a.inv = b->inv;
     a.tile = g.sched.tile;

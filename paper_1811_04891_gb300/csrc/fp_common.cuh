@@ -31,7 +31,10 @@ struct ElemBox {
     double blo[3];      // axis-aligned Bernstein-hull bounds minus pad
     double bhi[3];      //   ... plus pad
     double he;          // diagonal of the axis box spanned by the element's nodes
-    double spare;
+    double scale;       // power of two with |x - c| / scale < 1/2 over the nodes (digit form, see fp_tile.cuh)
+    double jscale[2];   // the same for the nodal values of dx/dr and dx/ds, in units of scale
+    double dev;         // largest distance of a node from its place in the affine frame, |y - xi| (infinity norm);
+                        //   infinite where it is not computed
 };
 
 // FP32 copy of ElemBox for the mixed form's screen, rounded outward with

@@ -159,7 +159,8 @@ __global__ void k_hull2(int n, int64_t E, const double* __restrict__ coords, con
         bx.Ai[3] = Ai[2]; bx.Ai[4] = Ai[3];
         bx.Ai[8] = 1.0;
         bx.he = he;
-        bx.spare = 0.0;
+        bx.scale = bx.jscale[0] = bx.jscale[1] = 1.0;
+        bx.dev = INFINITY;
         boxes[e] = bx;
         nodebox[6 * e + 0] = lo[0]; nodebox[6 * e + 1] = lo[1]; nodebox[6 * e + 2] = 0.0;
         nodebox[6 * e + 3] = hi[0]; nodebox[6 * e + 4] = hi[1]; nodebox[6 * e + 5] = 0.0;

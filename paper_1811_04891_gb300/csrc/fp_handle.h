@@ -30,6 +30,7 @@ struct fp_handle {
     double* coords = nullptr;      // [3][E][n3]
     float* coords32 = nullptr;     // [3][E][n3] element-local FP32 (mixed form)
     float* coords32lo = nullptr;   // [3][E][n3] low parts: (x - c) - coords32 (mixed form)
+    unsigned char* digits = nullptr;   // [E][tile_digits_bytes(n)] node digits (hexahedra, orders of the tile kernels)
     int32_t* sub = nullptr;        // [E]
     double* dist = nullptr;        // [E][n3] or null
     fpg::ElemBox* boxes = nullptr;      // [E]
@@ -50,7 +51,9 @@ struct fp_handle {
     int32_t* order = nullptr;
     double* pres = nullptr;
     double* prst = nullptr;
-    double2* pstate = nullptr;     // FP64 form: state of solves paused by the first Newton pass
+    double2* pstate = nullptr;     // state of solves paused by the first Newton pass (see keeps_state)
+    int32_t* pause_list = nullptr; // their list (orders of the tile kernels)
+    float* jst = nullptr;          // [9][cap] mixed form: Jacobians between its two launches
     int32_t* inv = nullptr;        // [cap] sorted position of each pair slot (hexahedral handles)
     int32_t* h_total = nullptr;    // pinned host word for the pair count
     // geometry scratch kept for fp_update_coords (moving meshes)

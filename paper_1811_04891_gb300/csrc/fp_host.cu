@@ -189,13 +189,26 @@ void release(fp_handle* h)
     h->ev_free.clear();
     dfree(h->stats);
     dfree(h->band);
-    dfree(h->coords); dfree(h->coords32); dfree(h->coords32lo); dfree(h->sub); dfree(h->dist); dfree(h->boxes); dfree(h->boxes32);
+    dfree(h->coords); dfree(h->digits); dfree(h->coords32); dfree(h->coords32lo); dfree(h->sub); dfree(h->dist); dfree(h->boxes); dfree(h->boxes32);
     dfree(h->cell_start); dfree(h->cell_elems); dfree(h->ecount); dfree(h->estart); dfree(h->escan_tmp);
     dfree(h->cnt); dfree(h->smask); dfree(h->off); dfree(h->scan_tmp); dfree(h->pair_elem); dfree(h->pair_pt);
-    dfree(h->order); dfree(h->pres); dfree(h->prst); dfree(h->pstate); dfree(h->inv);
-    dfree(h->binv); dfree(h->nodebox); dfree(h->red); dfree(h->hcnt); dfree(h->htmp); dfree(h->flag);
+    dfree(h->order); dfree(h->pres); dfree(h->prst); dfree(h->pstate); dfree(h->inv); dfree(h->pause_list);
+    dfree(h->jst); dfree(h->binv); dfree(h->nodebox); dfree(h->red); dfree(h->hcnt); dfree(h->htmp); dfree(h->flag);
     if (h->h_total) cudaFreeHost(h->h_total);
     h->h_total = nullptr;
+}
+
+// whether finds on this handle pause solves after a first Newton pass (the
+// FP64 form, and both forms with tile kernels); bytes per pair that takes
+bool keeps_state(const fp_handle* h)
+{
+    return h->dim == 3 && (h->opts.precision == FP_PREC_FP64 || is_tile_order(h->n, h->opts.precision == FP_PREC_MIXED));
+}
+
+int64_t pause_bytes(const fp_handle* h)
+{
+    const bool tile = h->dim == 3 && is_tile_order(h->n, h->opts.precision == FP_PREC_MIXED);
+    return (keeps_state(h) ? 16 : 0) + (tile ? 4 : 0) + (tile && h->opts.precision == FP_PREC_MIXED ? 36 : 0);
 }
 
 fp_status grow_points(fp_handle* h, int64_t P)
@@ -221,14 +234,17 @@ fp_status grow_pairs(fp_handle* h, int64_t np)
     int64_t cap = std::max<int64_t>(np + np / 4, 2048);
     cudaDeviceSynchronize();
     dfree(h->pair_elem); dfree(h->pair_pt); dfree(h->order); dfree(h->pres); dfree(h->prst); dfree(h->pstate);
-    dfree(h->inv);
-    const bool two_pass = h->dim == 3 && h->opts.precision == FP_PREC_FP64;
+    dfree(h->inv); dfree(h->pause_list); dfree(h->jst);
+    const bool tile = h->dim == 3 && is_tile_order(h->n, h->opts.precision == FP_PREC_MIXED), two_pass = keeps_state(h);
+    const bool mixed = h->opts.precision == FP_PREC_MIXED;
     cudaError_t e;
     if ((e = dalloc(&h->pair_elem, cap)) != cudaSuccess || (e = dalloc(&h->pair_pt, cap)) != cudaSuccess ||
         (e = dalloc(&h->order, cap)) != cudaSuccess || (e = dalloc(&h->pres, cap)) != cudaSuccess ||
         (e = dalloc(&h->prst, 3 * cap)) != cudaSuccess ||
         (h->dim == 3 && (e = dalloc(&h->inv, cap)) != cudaSuccess) ||
-        (two_pass && (e = dalloc(&h->pstate, cap)) != cudaSuccess)) {
+        (two_pass && (e = dalloc(&h->pstate, cap)) != cudaSuccess) ||
+        (tile && (e = dalloc(&h->pause_list, cap)) != cudaSuccess) ||
+        (tile && mixed && (e = dalloc(&h->jst, 9 * cap)) != cudaSuccess)) {
         h->cap_pairs = 0;
         return cuda_fail(h, e, "workspace (pairs)");
     }
@@ -403,14 +419,22 @@ fp_status build_geometry(fp_handle* h, cudaStream_t s, bool default_dist)
         h->dist_default = true;
     }
 
+    // node digits of the tile kernels, with each element's scale and affine deviation
+    const bool mixed = o.precision == FP_PREC_MIXED;
+    if (h->dim == 3 && is_tile_order(n, mixed)) {
+        if (!h->digits) GK(dalloc(&h->digits, (size_t)E * tile_digits_bytes(n, mixed)), "alloc digits");
+        GK(launch_digits(n, mixed, E, h->coords, h->boxes, h->digits, h->tab, s), "digits");
+    }
+
     // mixed form: element-local FP32 geometry
     if (o.precision == FP_PREC_MIXED) {
         const size_t ncoord = (size_t)3 * E * n3;
         if (!h->coords32) GK(dalloc(&h->coords32, ncoord), "alloc coords32");
-        if (!h->coords32lo) GK(dalloc(&h->coords32lo, ncoord), "alloc coords32lo");
+        const bool lo = !is_tile_order(n, true);
+        if (lo && !h->coords32lo) GK(dalloc(&h->coords32lo, ncoord), "alloc coords32lo");
         if (!h->boxes32) GK(dalloc(&h->boxes32, E), "alloc boxes32");
         GK(launch_local32(n, E, h->coords, h->boxes, h->coords32, s), "local32");
-        GK(launch_local32lo(n, E, h->coords, h->boxes, h->coords32, h->coords32lo, s), "local32lo");
+        if (lo) GK(launch_local32lo(n, E, h->coords, h->boxes, h->coords32, h->coords32lo, s), "local32lo");
         GK(launch_box32(E, h->boxes, h->boxes32, s), "box32");
     }
 #undef GK
@@ -587,6 +611,7 @@ static fp_status find_impl(fp_handle* h, int64_t P, const double* pts, const int
     a.cell_start = h->cell_start; a.cell_elems = h->cell_elems;
     a.cnt = h->cnt; a.off = h->off; a.ecount = h->ecount; a.estart = h->estart; a.scan_tmp = h->scan_tmp;
     a.smask = h->dim == 3 ? h->smask : nullptr;
+    a.digits = h->digits;
     a.code = code; a.osub = sub; a.oelem = elem; a.rst = rst; a.dist2 = dist2;
     a.eval = ev;
     a.stats = h->prof ? h->stats : nullptr;
@@ -621,6 +646,7 @@ static fp_status find_impl(fp_handle* h, int64_t P, const double* pts, const int
     a.pair_elem = h->pair_elem; a.pair_pt = h->pair_pt; a.order = h->order;
     a.pres = h->pres; a.prst = h->prst; a.cap = h->cap_pairs; a.pstate = h->pstate;
     a.inv = d2 ? nullptr : h->inv;
+    a.pause_list = h->pause_list; a.jst = h->jst;
     if (npairs > 0) {
         err = d2 ? find_emit2(a, s) : find_emit(a, s);
         if (err != cudaSuccess) return cuda_fail(h, err, "fp_find emit");
@@ -630,7 +656,7 @@ static fp_status find_impl(fp_handle* h, int64_t P, const double* pts, const int
         h->ev_pend[PROF_SCREEN].push_back({scr0, scr1});
     }
     const int block = h->opts.points_per_block > 0 ? h->opts.points_per_block
-                                                   : (d2 ? kDefaultBlock : kDefaultBlockFind3);
+                                                   : (d2 || is_tile_order(h->n, h->opts.precision == FP_PREC_MIXED) ? kDefaultBlock : kDefaultBlockFind3);
     err = d2 ? find_solve2(a, npairs, h->tab, fp, block, s) : find_solve(a, npairs, h->tab, fp, block, s);
     if (h->prof) {
         if (npairs > 0) {
@@ -763,7 +789,9 @@ struct fp_workspace {
     int32_t *pair_elem = nullptr, *pair_pt = nullptr, *order = nullptr;
     int32_t *ecount = nullptr, *estart = nullptr;
     double *pres = nullptr, *prst = nullptr;
-    double2* pstate = nullptr;  // FP64 form: state of solves paused by the first Newton pass
+    double2* pstate = nullptr;  // state of solves paused by the first Newton pass (see keeps_state)
+    int32_t* pause_list = nullptr;   // their list (orders of the tile kernels)
+    float* jst = nullptr;            // [9][max_pairs] mixed form: Jacobians between its two launches
     int32_t* inv = nullptr;     // sorted position of each pair slot
 };
 
@@ -771,7 +799,7 @@ static void ws_release(fp_workspace* w)
 {
     dfree(w->cnt); dfree(w->smask); dfree(w->off); dfree(w->scan_tmp); dfree(w->pair_elem); dfree(w->pair_pt);
     dfree(w->order); dfree(w->ecount); dfree(w->estart); dfree(w->pres); dfree(w->prst); dfree(w->pstate);
-    dfree(w->inv);
+    dfree(w->inv); dfree(w->pause_list); dfree(w->jst);
 }
 
 fp_status fp_workspace_create(const fp_handle* h, int64_t max_points, int64_t max_pairs, fp_workspace** out)
@@ -799,7 +827,9 @@ fp_status fp_workspace_create(const fp_handle* h, int64_t max_points, int64_t ma
         (e = dalloc(&w->order, max_pairs)) != cudaSuccess || (e = dalloc(&w->ecount, h->E)) != cudaSuccess ||
         (e = dalloc(&w->estart, h->E + 1)) != cudaSuccess || (e = dalloc(&w->pres, max_pairs)) != cudaSuccess ||
         (e = dalloc(&w->prst, 3 * max_pairs)) != cudaSuccess || (e = dalloc(&w->inv, max_pairs)) != cudaSuccess ||
-        (h->opts.precision == FP_PREC_FP64 && (e = dalloc(&w->pstate, max_pairs)) != cudaSuccess)) {
+        (keeps_state(h) && (e = dalloc(&w->pstate, max_pairs)) != cudaSuccess) ||
+        (is_tile_order(h->n, h->opts.precision == FP_PREC_MIXED) && (e = dalloc(&w->pause_list, max_pairs)) != cudaSuccess) ||
+        (is_tile_order(h->n, h->opts.precision == FP_PREC_MIXED) && h->opts.precision == FP_PREC_MIXED && (e = dalloc(&w->jst, 9 * max_pairs)) != cudaSuccess)) {
         ws_release(w);
         delete w;
         return e == cudaErrorMemoryAllocation ? FP_ERR_OOM : FP_ERR_CUDA;
@@ -815,7 +845,7 @@ fp_status fp_workspace_bytes(const fp_handle* h, int64_t max_points, int64_t max
     if (max_pairs <= 0) max_pairs = 2 * max_points;
     if (max_pairs >= (int64_t(1) << 31)) return FP_ERR_INVALID_ARG;
     *bytes = 4 * max_points + 4 * max_points + 4 * (max_points + 1) + 4 * std::max(scan_tmp_elems(max_points), scan_tmp_elems(h->E)) +
-             max_pairs * (4 + 4 + 4 + 4 + 8 + 24 + (h->opts.precision == FP_PREC_FP64 ? 16 : 0)) + 4 * h->E +
+             max_pairs * (4 + 4 + 4 + 4 + 8 + 24 + pause_bytes(h)) + 4 * h->E +
              4 * (h->E + 1);
     return FP_OK;
 }
@@ -888,9 +918,11 @@ static fp_status find_ws_impl(fp_handle* h, fp_workspace* w, int64_t P, const do
     a.cell_start = h->cell_start; a.cell_elems = h->cell_elems;
     a.cnt = w->cnt; a.off = w->off; a.scan_tmp = w->scan_tmp; a.ecount = w->ecount; a.estart = w->estart;
     a.smask = w->smask;
+    a.digits = h->digits;
     a.pair_elem = w->pair_elem; a.pair_pt = w->pair_pt; a.order = w->order; a.pres = w->pres; a.prst = w->prst;
     a.pstate = w->pstate;
     a.inv = w->inv;
+    a.pause_list = w->pause_list; a.jst = w->jst;
     a.cap = w->max_pairs;
     a.persistent_blocks = w->persistent_blocks;
     a.code = code; a.osub = sub; a.oelem = elem; a.rst = rst; a.dist2 = dist2;
@@ -1170,13 +1202,14 @@ fp_status fp_memory(const fp_handle* h, int64_t* resident, int64_t* workspace)
                     4 * h->ncell_cap + 4 * scan_tmp_elems(h->ncell_cap) + 4 * h->nnz_cap + 8 * (int64_t)h->n * h->n +
                     96 * (int64_t)h->nred + 4 * h->E + 4 * (h->E + 1);
         if (h->dist) b += 8 * h->E * n3;
-        if (h->coords32) b += 8 * nc + (int64_t)sizeof(ElemBox32) * h->E;
+        if (h->coords32) b += (h->coords32lo ? 8 : 4) * nc + (int64_t)sizeof(ElemBox32) * h->E;
+        if (h->digits) b += tile_digits_bytes(h->n, h->opts.precision == FP_PREC_MIXED) * h->E;
         *resident = b;
     }
     if (workspace)
         *workspace = 4 * h->cap_pts + 4 * h->cap_pts + 4 * (h->cap_pts + 1) +
                      4 * (h->cap_pts > 0 ? std::max(scan_tmp_elems(h->cap_pts), scan_tmp_elems(h->E)) : 0) +
-                     h->cap_pairs * (4 + 4 + 4 + 8 + 24 + (h->pstate ? 16 : 0) + (h->inv ? 4 : 0));
+                     h->cap_pairs * (4 + 4 + 4 + 8 + 24 + (h->pstate ? 16 : 0) + (h->pause_list ? 4 : 0) + (h->jst ? 36 : 0) + (h->inv ? 4 : 0));
     return FP_OK;
 }
 

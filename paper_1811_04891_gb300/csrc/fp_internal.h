@@ -112,7 +112,7 @@ struct FindArgs {
     int tile;                     // sorted positions per work item (0: one block's worth)
     int32_t* fb_count;            // mixed form, batch groups: fallback counter and list (group slice
     int32_t* fb_list;             //   from the group's first sorted position)
-    double2* pstate;              // FP64 form: [cap] state of solves paused by the first pass (null: one pass)
+    double2* pstate;              // [cap] state of solves paused by the first Newton pass (null: one pass)
     // outputs
     int32_t* code;
     int32_t* osub;
@@ -122,7 +122,34 @@ struct FindArgs {
     uint32_t* smask = nullptr;    // [P] screen: candidates that passed the count pass, by bit of the
                                   //   cell list (bit 31: list too long, test again); null = test again
     int batch = 0;                // 1: a batch group (its own FP64 first-pass budget)
+    const unsigned char* digits = nullptr;   // the elements' node digits (orders of the tile kernels)
+    int32_t* pause_list = nullptr;           // [cap] tile kernels: paused solves (with pstate); null: one pass
+    float* jst = nullptr;                    // [9][cap] mixed form: Jacobians kept between its two launches
+    int32_t* pause_count = nullptr;          // batch groups: their number (otherwise the second scan scratch word)
 };
+
+// Tensor-core tile kernels (fp_tile.cuh) of the Newton stage: their orders,
+// the bytes of an element's node digits (0 for other orders) and the kernel
+// that lays them out (also boxes[].scale, jscale and dev).
+//
+// The order decides alone, never the number of points, so that every entry
+// point gives a pair the same bits.  Lower orders have too little to contract,
+// higher ones more columns than a warp's accumulators hold.  FP64 form: faster
+// at every density for N = 3..9 (1.5 to 8 times).  Mixed form, fp_find in us,
+// one thread per pair / tiles, at 0.7, 5 and 600 points per element:
+//   N = 3  149/143  159/171   922/ 707     N = 4  183/159  193/190  1249/ 855
+//   N = 5  197/171  205/245  1438/1114     N = 6  249/198  274/280  1959/1318
+//   N = 7  281/183  315/276  2113/1289     N = 8  407/279  444/469  3178/2102
+//   N = 9  489/331  599/594  3617/2807
+// N = 3 and 5 lose 8 and 20 % at a few points per element (n^2 = 16 and 36
+// fill the k16 steps and n their columns badly) and keep one thread per pair.
+constexpr bool is_tile_order(int n, bool mixed)
+{
+    return mixed ? n == 5 || (n >= 7 && n <= 10) : n >= 4 && n <= 10;
+}
+int64_t tile_digits_bytes(int n, bool mixed);
+cudaError_t launch_digits(int n, bool mixed, int64_t E, const double* coords, ElemBox* boxes, unsigned char* dig,
+                          const BasisTab& tab, cudaStream_t s);
 cudaError_t find_count(const FindArgs& a, const BasisTab& tab, const FindParams& fp, cudaStream_t s);
 cudaError_t find_screen_count(const FindArgs& a, cudaStream_t s);   // counts only, no scan
 cudaError_t find_emit(const FindArgs& a, cudaStream_t s);

@@ -200,7 +200,8 @@ __global__ void k_hull(int n, int64_t E, const double* __restrict__ coords,
         }
         for (int q = 0; q < 9; ++q) bx.Ai[q] = Ai[q];
         bx.he = he;
-        bx.spare = 0.0;
+        bx.scale = bx.jscale[0] = bx.jscale[1] = 1.0;
+        bx.dev = INFINITY;
         boxes[e] = bx;
         for (int a = 0; a < 3; ++a) {
             nodebox[6 * e + a] = lo[a];

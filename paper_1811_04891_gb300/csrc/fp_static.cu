@@ -134,6 +134,7 @@ extern "C" fp_status fp_find_static(fp_handle* h, int64_t P, const double* pts, 
     a.dist = h->nsub > 1 ? h->dist : nullptr;
     a.boxes = h->boxes; a.boxes32 = h->boxes32; a.grid = &h->grid;
     a.cell_start = h->cell_start; a.cell_elems = h->cell_elems;
+    a.digits = h->digits;
     a.cnt = reinterpret_cast<int32_t*>(b + kOffCnt);
     a.off = reinterpret_cast<int32_t*>(b + kOffOff);
     a.scan_tmp = reinterpret_cast<int32_t*>(b + kOffScan);
