@@ -163,9 +163,10 @@ struct RankBatch {
     __device__ __forceinline__ double he(int e) const { return he_all[e]; }
     __device__ __forceinline__ int sub(int e) const { return sub_all[e]; }
     __device__ __forceinline__ bool has_dist() const { return grp[g].dist != nullptr; }
-    __device__ double delta(int e, int64_t q) const
+    __device__ __forceinline__ int tag() const { return g; }
+    __device__ double delta(int tag, int e, int64_t q) const
     {
-        const BRankGroup G = grp[g];
+        const BRankGroup G = grp[tag];
         const int n = G.n;
         double hr[NMAX], hs[NMAX], ht[NMAX];
         lagrange_rt(n, G.tab->xi, G.tab->ci, A.prst[q], hr);
@@ -187,12 +188,11 @@ struct RankBatch {
     __device__ __forceinline__ int elem_out(int e) const { return e - ebase_inst; }
 };
 
-__global__ void __launch_bounds__(128) k_rank_batch(RankArgs A, FindParams fp, int ninst, const BRankInst* inst,
+__global__ void __launch_bounds__(kRankThreads) k_rank_batch(RankArgs A, FindParams fp, int ninst, const BRankInst* inst,
                                                     const int64_t* p0, const double* he_all, const int32_t* sub_all,
                                                     const BRankGroup* grp)
 {
     const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (p >= A.P) return;
     int lo = 0, hi = ninst;
     while (hi - lo > 1) {
         const int mid = (lo + hi) >> 1;
@@ -203,7 +203,7 @@ __global__ void __launch_bounds__(128) k_rank_batch(RankArgs A, FindParams fp, i
     FindParams f = fp;
     f.band = I.band;
     const RankBatch C{he_all, sub_all, grp, A, I.ebase, I.grp};
-    rank_point<3>(A, f, C, p);
+    rank_point<3>(A, f, C, p, p < A.P);
 }
 
 __global__ void k_fill_he(int64_t E, const ElemBox* __restrict__ boxes, double* __restrict__ he)
@@ -618,7 +618,7 @@ static cudaError_t batch_run(fp_batch* b, const double* pts, int32_t* code, int3
         ra.band = b->band;
         ra.inv = b->inv;
         FindParams fp = b->groups[0].fp;
-        k_rank_batch<<<(unsigned)((P + 127) / 128), 128, 0, s>>>(ra, fp, b->ninst, b->d_rinst, b->d_p0, b->he_all,
+        k_rank_batch<<<(unsigned)((P + kRankThreads - 1) / kRankThreads), kRankThreads, 0, s>>>(ra, fp, b->ninst, b->d_rinst, b->d_p0, b->he_all,
                                                                 b->sub_all, b->d_rgrp);
         count_launch();
         if ((e = cudaGetLastError()) != cudaSuccess) return e;

@@ -483,7 +483,7 @@ static cudaError_t solve_n(const FindArgs& a, int64_t npairs, const BasisTab& ta
     ra.band = a.band;
     ra.inv = a.inv;
     if (a.ev[4]) cudaEventRecord(a.ev[4], s);
-    k_rank<n, 3><<<(unsigned)((a.P + 127) / 128), 128, 0, s>>>(ra, fp, tab);
+    k_rank<n, 3><<<(unsigned)((a.P + kRankThreads - 1) / kRankThreads), kRankThreads, 0, s>>>(ra, fp, tab);
     count_launch();
     if (a.ev[5]) cudaEventRecord(a.ev[5], s);
     cudaError_t err = cudaGetLastError();
