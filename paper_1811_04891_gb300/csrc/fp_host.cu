@@ -277,9 +277,11 @@ fp_status build_geometry(fp_handle* h, cudaStream_t s, bool default_dist)
         h->nred = (int)std::min<int64_t>(1024, (E + 255) / 256);
         GK(dalloc(&h->red, 12 * h->nred), "alloc red");
     }
-    if (h->dim == 2)
-        GK(launch_hull2(n, E, h->coords, h->binv, o.tol_border, h->pad_conv, h->boxes, h->nodebox, s), "hull");
-    else
+    if (h->dim == 2) {
+        if (!h->coords32) GK(dalloc(&h->coords32, (size_t)2 * E * n3), "alloc coords32");
+        GK(launch_hull2(n, E, h->coords, h->binv, o.tol_border, h->pad_conv, h->boxes, h->nodebox, h->coords32, h->tab, s),
+           "hull");
+    } else
         GK(launch_hull(n, E, h->coords, h->binv, o.tol_border, h->pad_conv, h->boxes, h->nodebox, s), "hull");
     GK(launch_reduce_boxes(E, h->boxes, h->nodebox, h->red, h->nred, s), "reduce boxes");
     std::vector<double> red(12 * h->nred);
@@ -1202,7 +1204,7 @@ fp_status fp_memory(const fp_handle* h, int64_t* resident, int64_t* workspace)
                     4 * h->ncell_cap + 4 * scan_tmp_elems(h->ncell_cap) + 4 * h->nnz_cap + 8 * (int64_t)h->n * h->n +
                     96 * (int64_t)h->nred + 4 * h->E + 4 * (h->E + 1);
         if (h->dist) b += 8 * h->E * n3;
-        if (h->coords32) b += (h->coords32lo ? 8 : 4) * nc + (int64_t)sizeof(ElemBox32) * h->E;
+        if (h->coords32) b += (h->coords32lo ? 8 : 4) * nc + (h->boxes32 ? (int64_t)sizeof(ElemBox32) * h->E : 0);
         if (h->digits) b += tile_digits_bytes(h->n, h->opts.precision == FP_PREC_MIXED) * h->E;
         *resident = b;
     }

@@ -180,7 +180,8 @@ cudaError_t find_sort(const FindArgs& a, int64_t npairs, cudaStream_t s);
 
 // 2D quadrilateral variant (fp_find2.cu): coords [2][E][n^2], pts / rst [2][P]
 cudaError_t launch_hull2(int n, int64_t E, const double* coords, const double* binv, double pad_border,
-                         double pad_conv, ElemBox* boxes, double* nodebox, cudaStream_t s);
+                         double pad_conv, ElemBox* boxes, double* nodebox, float* c32, const BasisTab& tab,
+                         cudaStream_t s);
 // default D^k from the boundary edges of each subdomain; *too_large when the
 // node x boundary-node pairs exceed max_pairs (nothing computed then)
 cudaError_t launch_dist_default2(int n, int64_t E, const double* coords, const int32_t* sub, const HashGrid& g,
