@@ -3,11 +3,211 @@
 // in FP64; quiet NaN for points that were not found.
 #include <algorithm>
 #include <climits>
+#include <type_traits>
 
 #include "fp_common.cuh"
 #include "fp_internal.h"
 
 namespace fpg {
+
+// ---------------------------------------------------------------------------
+// Evaluation by planes: the n planes k of a point's element are contracted by
+// n neighbouring lanes, then one lane per field adds them up over k.  Every
+// value takes the operations of the one-thread form (contract, contract_df)
+// in the same order, so the two agree bit for bit.
+//
+// Up to some 10^5 values the one-thread form leaves the GPU nearly empty: its
+// time is that of one thread's chain of n^3 terms per field, with every load
+// a row of its own.  By planes the chain is n times shorter and a warp works
+// on few elements at a time.  The basis is evaluated once per group, one
+// direction a lane (one FP64 basis a warp instead of three).
+// ---------------------------------------------------------------------------
+template <int n> constexpr int kPlaneGroup = n <= 2 ? 2 : n <= 4 ? 4 : n <= 8 ? 8 : 16;   // lanes of a point
+
+struct PlanesDf {                       // posted fields
+    using W = float2;                   // weights and plane sums: float pairs
+    using V = float2;
+    static __device__ __forceinline__ W weight(double h)
+    {
+        const df a = df_split(h);
+        return make_float2(a.hi, a.lo);
+    }
+    template <int n>
+    static __device__ __forceinline__ W plane(const V* __restrict__ F, const W* __restrict__ w)
+    {
+        float rh[n], rl[n];
+#pragma unroll
+        for (int i = 0; i < n; ++i) {
+            rh[i] = w[i].x;
+            rl[i] = w[i].y;
+        }
+        df c = {0.0f, 0.0f};
+#pragma unroll 2
+        for (int j = 0; j < n; ++j) {
+            const W s = w[n + j];
+            df_fma_acc(c, row_df<n>(F + n * j, rh, rl), s.x, s.y);
+        }
+        df_norm(c);
+        return make_float2(c.hi, c.lo);
+    }
+    template <int n>
+    static __device__ __forceinline__ double sum(const W* __restrict__ c, const W* __restrict__ t)
+    {
+        df acc = {0.0f, 0.0f};
+#pragma unroll
+        for (int k = 0; k < n; ++k) df_fma_acc(acc, df{c[k].x, c[k].y}, t[k].x, t[k].y);
+        return (double)acc.hi + (double)acc.lo;
+    }
+};
+
+struct PlanesF64 {
+    using W = double;
+    using V = double;
+    static __device__ __forceinline__ W weight(double h) { return h; }
+    template <int n>
+    static __device__ __forceinline__ W plane(const V* __restrict__ F, const W* __restrict__ w)
+    {
+        double hr[n];
+#pragma unroll
+        for (int i = 0; i < n; ++i) hr[i] = w[i];
+        double c = 0.0;
+#pragma unroll 2
+        for (int j = 0; j < n; ++j) {
+            double v[n];
+            load_row<n>(F + n * j, v);
+            double u = 0.0;
+#pragma unroll
+            for (int i = 0; i < n; ++i) u = fma(hr[i], v[i], u);
+            c = fma(w[n + j], u, c);
+        }
+        return c;
+    }
+    template <int n>
+    static __device__ __forceinline__ double sum(const W* __restrict__ c, const W* __restrict__ t)
+    {
+        double acc = 0.0;
+#pragma unroll
+        for (int k = 0; k < n; ++k) acc = fma(t[k], c[k], acc);
+        return acc;
+    }
+};
+
+template <int n, class O>
+struct PlaneSm {
+    static constexpr int G = kPlaneGroup<n>;
+    typename O::W w[32 / G][3 * n];     // basis values in r, s, t
+    typename O::W c[32 / G][G * n];     // plane sums of up to G fields
+};
+
+// the basis values at (r0, r1, r2) = R(0), R(1), R(2)
+template <int n, class O, class R>
+__device__ __forceinline__ void plane_basis(typename O::W* w, int g, const BasisTab& tab, R&& r)
+{
+    for (int d = g; d < 3; d += kPlaneGroup<n>) {
+        double h[n];
+        lagrange_h<n, double>(tab.xi, tab.ci, r(d), h);
+#pragma unroll
+        for (int i = 0; i < n; ++i) w[d * n + i] = O::weight(h[i]);
+    }
+}
+
+// the F fields at a group's point (w set); every lane of the warp takes part
+template <int n, class O>
+__device__ __forceinline__ void plane_values(const typename O::W* w, typename O::W* c, int g, bool ok,
+                                             const typename O::V* __restrict__ fields, int64_t E, int F, int e,
+                                             double* __restrict__ out, int64_t P, int64_t p)
+{
+    constexpr int G = kPlaneGroup<n>, n2 = n * n;
+    for (int f0 = 0; f0 < F; f0 += G) {
+        const int nf = min(G, F - f0);
+        __syncwarp();
+        if (ok && g < n)
+            for (int f = 0; f < nf; ++f)
+                c[f * n + g] = O::template plane<n>(fields + (((int64_t)(f0 + f) * E + e) * n + g) * n2, w);
+        __syncwarp();
+        if (ok && g < nf) out[(int64_t)(f0 + g) * P + p] = O::template sum<n>(c + g * n, w + 2 * n);
+    }
+}
+
+// points in the caller's order (k_eval, k_eval_df), or posted points (basis
+// and pe: k_eval_points_df)
+template <int n, class O>
+__global__ void __launch_bounds__(128) k_eval_planes(int64_t E, int64_t P, const int32_t* __restrict__ code,
+                                                     const int32_t* __restrict__ elem, const double* __restrict__ rst,
+                                                     const float* __restrict__ basis, int F,
+                                                     const typename O::V* __restrict__ fields, double* __restrict__ out,
+                                                     BasisTab tab)
+{
+    constexpr int G = kPlaneGroup<n>;
+    __shared__ PlaneSm<n, O> sm[4];
+    PlaneSm<n, O>& S = sm[threadIdx.x >> 5];
+    const int lane = threadIdx.x & 31, g = lane % G, gr = lane / G;
+    const int64_t p = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / G;
+    const int e = p < P ? elem[p] : -1;
+    const bool ok = e >= 0 && e < E && (!code || (code[p] != FP_CODE_NOT_FOUND && code[p] != FP_CODE_RETRY));
+    typename O::W* w = S.w[gr];
+    if (ok) {
+        if constexpr (sizeof(typename O::V) == sizeof(float2) && !std::is_same_v<O, PlanesF64>) {
+            if (basis) {
+                for (int i = g; i < n; i += G)
+#pragma unroll
+                    for (int d = 0; d < 3; ++d)
+                        w[d * n + i] = make_float2(__ldg(basis + ((int64_t)(2 * d) * n + i) * P + p),
+                                                   __ldg(basis + ((int64_t)(2 * d + 1) * n + i) * P + p));
+            } else {
+                plane_basis<n, O>(w, g, tab, [&](int d) { return rst[d * P + p]; });
+            }
+        } else {
+            plane_basis<n, O>(w, g, tab, [&](int d) { return rst[d * P + p]; });
+        }
+    } else if (p < P) {
+        for (int f = g; f < F; f += G) out[(int64_t)f * P + p] = __longlong_as_double(0x7ff8000000000000ULL);
+    }
+    plane_values<n, O>(w, S.c[gr], g, ok, fields, E, F, e, out, P, p);
+}
+
+struct EvalPairsArgs {
+    int64_t E, P, cap;
+    const int32_t* dcount;
+    const int32_t* order;
+    const int32_t* pair_elem;
+    const int32_t* pair_pt;
+    const double* prst;
+    EvalSpec ev;
+    const int32_t* s_lo;      // batch groups: the group's sorted positions [*s_lo, *s_hi)
+    const int32_t* s_hi;
+    int32_t ebase;            // batch groups: subtracted from pair_elem
+    int walk;                 // pair results at sorted positions (else at pair slots)
+};
+
+// winning pairs in the find's element-sorted order (k_eval_pairs)
+template <int n, class O>
+__global__ void __launch_bounds__(128) k_eval_pairs_planes(EvalPairsArgs A, const typename O::V* __restrict__ fields,
+                                                           BasisTab tab)
+{
+    constexpr int G = kPlaneGroup<n>;
+    __shared__ PlaneSm<n, O> sm[4];
+    PlaneSm<n, O>& S = sm[threadIdx.x >> 5];
+    const int lane = threadIdx.x & 31, g = lane % G, gr = lane / G;
+    const int64_t t = *A.dcount, s1 = t < A.cap ? t : A.cap;
+    const int64_t step = (int64_t)gridDim.x * 4 * (32 / G);
+    for (int64_t base = ((int64_t)blockIdx.x * 4 + (threadIdx.x >> 5)) * (32 / G); base < s1; base += step) {
+        const int64_t s = base + gr;
+        int32_t p = -1;
+        int e = 0;
+        if (s < s1) {
+            const int32_t q = A.order[s];
+            p = A.pair_pt[q];
+            if (p >= 0) {                                 // the point's winning pair
+                e = A.pair_elem[q];
+                const int64_t w = A.walk ? s : q;
+                plane_basis<n, O>(S.w[gr], g, tab, [&](int d) { return A.prst[d * A.cap + w]; });
+            }
+        }
+        plane_values<n, O>(S.w[gr], S.c[gr], g, p >= 0, fields, A.E, A.ev.F, e, A.ev.out, A.P, p);
+        __syncwarp();                                     // the next pairs overwrite the basis
+    }
+}
 
 struct EvalArgs {
     int64_t E;
@@ -48,18 +248,41 @@ __global__ void __launch_bounds__(128) k_eval(EvalArgs A, BasisTab tab)
 // calls with at most this many (point, field) values take one thread each
 constexpr int64_t kSplitEval = int64_t(1) << 21;
 
+// Calls with at most this many (point, field) values (fused: points) evaluate
+// by planes.  us, one thread per value / planes, N = 7: 2,000 values 38/16,
+// 10,000 values 40/22, 40,000 values 73/52 at random points; but where
+// neighbouring points share their element, 131,072 values take 49/141.
+// Sorted pairs, whole find and evaluation of 4 posted fields: 2,000 points
+// 259/188, 10,000 361/270, 40,000 418/435.
+constexpr int64_t kPlaneValues = 20000, kPlanePairs = 20000;
+
+// Calls with at most this many points take one thread per sorted pair and
+// field, at n = 6 and above: find and evaluation of 4 posted fields at N = 7,
+// 40,000 points 424 -> 383 us (N = 9 684 -> 640, FP64 fields 933 -> 902); with
+// 130,000 the basis of every field costs more than the threads give (642 ->
+// 679), at N = 3 already with 40,000 (196 -> 208).
+constexpr int64_t kSplitPairs = 65536;
+constexpr int kSplitFields = 16, kSplitMinN = 6;
+
+template <int n>
+static unsigned plane_grid(int64_t count)
+{
+    return (unsigned)((count * kPlaneGroup<n> + 127) / 128);
+}
+
 cudaError_t launch_eval(int n, int64_t E, int64_t P, const int32_t* code, const int32_t* elem, const double* rst,
                         int F, const double* fields, double* out, const BasisTab& tab, cudaStream_t s)
 {
     if (P == 0) return cudaSuccess;
     EvalArgs a{E, P, code, elem, rst, F, fields, out};
-    const bool split = P * F <= kSplitEval;
+    const bool split = P * F <= kSplitEval, planes = P * F <= kPlaneValues;
     const unsigned grid = (unsigned)(((split ? P * F : P) + 127) / 128);
     switch (n) {
-#define FP_CASE(NN)                                                  \
-    case NN:                                                         \
-        if (split) k_eval<NN, true><<<grid, 128, 0, s>>>(a, tab);    \
-        else k_eval<NN, false><<<grid, 128, 0, s>>>(a, tab);         \
+#define FP_CASE(NN)                                                                                           \
+    case NN:                                                                                                  \
+        if (planes) k_eval_planes<NN, PlanesF64><<<plane_grid<NN>(P), 128, 0, s>>>(E, P, code, elem, rst, nullptr, F, fields, out, tab); \
+        else if (split) k_eval<NN, true><<<grid, 128, 0, s>>>(a, tab);                                        \
+        else k_eval<NN, false><<<grid, 128, 0, s>>>(a, tab);                                                  \
         break;
         FP_CASE(2) FP_CASE(3) FP_CASE(4) FP_CASE(5) FP_CASE(6) FP_CASE(7) FP_CASE(8) FP_CASE(9)
         FP_CASE(10) FP_CASE(11) FP_CASE(12) FP_CASE(13) FP_CASE(14) FP_CASE(15) FP_CASE(16)
@@ -152,16 +375,22 @@ __global__ void k_points_basis(int64_t P, const int32_t* __restrict__ code, cons
     }
 }
 
+// One thread per (point, field).  A block takes one field at consecutive
+// points: interface nodes follow the faces, so these lie in one element, and
+// the lanes of a warp load the same row in one access instead of one per
+// field.  32,768 interface nodes, 4 fields, N = 7: 71 -> 49 us.
+__host__ __device__ __forceinline__ unsigned value_blocks(int64_t P) { return (unsigned)((P + 127) / 128); }
+
 template <int n>
 __global__ void __launch_bounds__(128) k_eval_points_df(int64_t E, int64_t P, int F, const int32_t* __restrict__ pe,
                                                         const float* __restrict__ basis,
                                                         const float2* __restrict__ fields, double* __restrict__ out)
 {
     constexpr int n3 = n * n * n;
-    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    const int64_t p = t / F;
+    const unsigned nb = value_blocks(P);
+    const int f = (int)(blockIdx.x / nb);
+    const int64_t p = (int64_t)(blockIdx.x - f * nb) * blockDim.x + threadIdx.x;
     if (p >= P) return;
-    const int f = (int)(t % F);
     const int e = pe[p];
     if (e < 0 || e >= E) {
         out[(int64_t)f * P + p] = __longlong_as_double(0x7ff8000000000000ULL);
@@ -223,10 +452,14 @@ cudaError_t launch_eval_points_df(int n, int64_t E, int64_t P, int F, const int3
                                   const float2* fields, double* out, cudaStream_t s)
 {
     if (P == 0) return cudaSuccess;
-    const unsigned grid = (unsigned)((P * F + 127) / 128);
+    const unsigned grid = value_blocks(P) * F;
+    const bool planes = P * F <= kPlaneValues;
     switch (n) {
-#define FP_CASE(NN) \
-    case NN: k_eval_points_df<NN><<<grid, 128, 0, s>>>(E, P, F, pe, basis, fields, out); break;
+#define FP_CASE(NN)                                                                                           \
+    case NN:                                                                                                  \
+        if (planes) k_eval_planes<NN, PlanesDf><<<plane_grid<NN>(P), 128, 0, s>>>(E, P, nullptr, pe, nullptr, basis, F, fields, out, BasisTab()); \
+        else k_eval_points_df<NN><<<grid, 128, 0, s>>>(E, P, F, pe, basis, fields, out);                      \
+        break;
         FP_CASE(2) FP_CASE(3) FP_CASE(4) FP_CASE(5) FP_CASE(6) FP_CASE(7) FP_CASE(8) FP_CASE(9)
         FP_CASE(10) FP_CASE(11) FP_CASE(12) FP_CASE(13) FP_CASE(14) FP_CASE(15) FP_CASE(16)
 #undef FP_CASE
@@ -241,12 +474,13 @@ cudaError_t launch_eval_df(int n, int64_t E, int64_t P, const int32_t* code, con
 {
     if (P == 0) return cudaSuccess;
     Eval2Args a{E, P, code, elem, rst, F, fields, out};
-    const bool split = P * F <= kSplitEval;
+    const bool split = P * F <= kSplitEval, planes = P * F <= kPlaneValues;
     const unsigned grid = (unsigned)(((split ? P * F : P) + 127) / 128);
     switch (n) {
 #define FP_CASE(NN)                                                     \
     case NN:                                                            \
-        if (split) k_eval_df<NN, true><<<grid, 128, 0, s>>>(a, tab);    \
+        if (planes) k_eval_planes<NN, PlanesDf><<<plane_grid<NN>(P), 128, 0, s>>>(E, P, code, elem, rst, nullptr, F, fields, out, tab); \
+        else if (split) k_eval_df<NN, true><<<grid, 128, 0, s>>>(a, tab);    \
         else k_eval_df<NN, false><<<grid, 128, 0, s>>>(a, tab);         \
         break;
         FP_CASE(2) FP_CASE(3) FP_CASE(4) FP_CASE(5) FP_CASE(6) FP_CASE(7) FP_CASE(8) FP_CASE(9)
@@ -301,23 +535,14 @@ __device__ __forceinline__ void eval_point_df(const float2* __restrict__ Fdf, in
         out[(int64_t)f * P + p] = contract_df<n>(Fdf + ((int64_t)f * E + e) * n3, rh, rl, sh, sl, th, tl);
 }
 
-struct EvalPairsArgs {
-    int64_t E, P, cap;
-    const int32_t* dcount;
-    const int32_t* order;
-    const int32_t* pair_elem;
-    const int32_t* pair_pt;
-    const double* prst;
-    EvalSpec ev;
-    const int32_t* s_lo;      // batch groups: the group's sorted positions [*s_lo, *s_hi)
-    const int32_t* s_hi;
-    int32_t ebase;            // batch groups: subtracted from pair_elem
-    int walk;                 // pair results at sorted positions (else at pair slots)
-};
 
+// one thread per winning pair, or (gridDim.y = F) one per pair and field
 template <int n, bool DF>
 __global__ void __launch_bounds__(128) k_eval_pairs(EvalPairsArgs A, BasisTab tab)
 {
+    constexpr int n3 = n * n * n;
+    const int nf = A.ev.F / (int)gridDim.y;
+    const int64_t f0 = (int64_t)blockIdx.y * nf;
     int64_t s0 = 0, s1;
     if (A.s_lo) {
         s0 = *A.s_lo;
@@ -334,9 +559,9 @@ __global__ void __launch_bounds__(128) k_eval_pairs(EvalPairsArgs A, BasisTab ta
         const int64_t w = A.walk ? s : q;
         const double r0 = A.prst[w], r1 = A.prst[A.cap + w], r2 = A.prst[2 * A.cap + w];
         if (DF)
-            eval_point_df<n>(A.ev.fdf, A.E, A.ev.F, e, r0, r1, r2, tab, A.ev.out, A.P, p);
+            eval_point_df<n>(A.ev.fdf + f0 * A.E * n3, A.E, nf, e, r0, r1, r2, tab, A.ev.out + f0 * A.P, A.P, p);
         else
-            eval_point_f64<n>(A.ev.f64, A.E, A.ev.F, e, r0, r1, r2, tab, A.ev.out, A.P, p);
+            eval_point_f64<n>(A.ev.f64 + f0 * A.E * n3, A.E, nf, e, r0, r1, r2, tab, A.ev.out + f0 * A.P, A.P, p);
     }
 }
 
@@ -428,12 +653,16 @@ cudaError_t launch_eval_pairs(int n, int64_t E, int64_t P, const int32_t* dcount
     const bool df = ev.fdf != nullptr;
     const int64_t stage_bytes = (int64_t)ev.F * n * n * n * (int64_t)sizeof(float2);
     const bool staged = df && ev.staged && stage_bytes <= kStageMaxBytes;
+    const bool planes = !s_lo && P <= kPlanePairs, split = !s_lo && P <= kSplitPairs && n >= kSplitMinN && ev.F <= kSplitFields;
+    const dim3 grid2(grid, split ? ev.F : 1);
     switch (n) {
 #define FP_CASE(NN)                                                                       \
     case NN:                                                                              \
-        if (staged) k_eval_pairs_staged<NN><<<grid, kStageTile, stage_bytes, s>>>(a, tab); \
-        else if (df) k_eval_pairs<NN, true><<<grid, 128, 0, s>>>(a, tab);                 \
-        else k_eval_pairs<NN, false><<<grid, 128, 0, s>>>(a, tab);                        \
+        if (planes && df) k_eval_pairs_planes<NN, PlanesDf><<<grid * kPlaneGroup<NN>, 128, 0, s>>>(a, ev.fdf, tab); \
+        else if (planes) k_eval_pairs_planes<NN, PlanesF64><<<grid * kPlaneGroup<NN>, 128, 0, s>>>(a, ev.f64, tab); \
+        else if (staged && !split) k_eval_pairs_staged<NN><<<grid, kStageTile, stage_bytes, s>>>(a, tab); \
+        else if (df) k_eval_pairs<NN, true><<<grid2, 128, 0, s>>>(a, tab);                \
+        else k_eval_pairs<NN, false><<<grid2, 128, 0, s>>>(a, tab);                       \
         break;
         FP_CASE(2) FP_CASE(3) FP_CASE(4) FP_CASE(5) FP_CASE(6) FP_CASE(7) FP_CASE(8) FP_CASE(9)
         FP_CASE(10) FP_CASE(11) FP_CASE(12) FP_CASE(13) FP_CASE(14) FP_CASE(15) FP_CASE(16)
