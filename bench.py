@@ -73,10 +73,9 @@ def work_for_order(n: int) -> dict:
 WORK = {"fp64": {"f64": SEED + K_ORACLE * ITER, "f32": 0.0, "f64acc": 0.0},
         "mixed": {"f64": 0.0, "f32": SEED + K_ORACLE * ITER, "f64acc": FINAL}}
 # DRAM bytes (read + written) per (point, candidate element) pair of the Newton
-# stage, from one-pass ncu captures of the stage at this full size
-# (dram__bytes_read.sum + dram__bytes_write.sum of k_newton_mixed, and of
-# k_newton + k_newton_resume, over the 10.24 M pairs of one launch).
-TRAFFIC_PER_PAIR = {"mixed": 622.0, "fp64": 620.0}
+# stage, from a one-pass ncu capture of its launches at this full size; empty:
+# not captured for the tensor-core kernels.
+TRAFFIC_PER_PAIR = {}
 HBM_FALLBACK_GBS = 6800.0
 
 
@@ -291,7 +290,7 @@ def roofline_form(form, P, F, kernel_ms, ms_per_step, peaks, hbm_gbs, pairs, coo
     fp64_view = P * (SEED + K_ORACLE * ITER + F * EVAL1) / p64
     return {"bound": "alu", "achieved": achieved / 1e12, "peak": peak / 1e12, "unit": unit,
             "frac": t_newton / kn, "traffic": None if traffic is None else traffic * pairs,
-            "kernel": "k_newton_mixed<8> + k_newton64_full<8>" if form == "mixed" else "k_newton<8>",
+            "kernel": "k_newton_tile<8> + k_newton64_full<8>" if form == "mixed" else "k_newton_tile<8>",
             "kernel_ms": kernel_ms["newton"], "units_per_launch": P, "work_unit": "located point (true element only)",
             "unit_work": w, "pairs_per_launch": pairs, "roofline_ms": 1e3 * t_newton,
             "peaks_tflops": {"p64": peaks["p64"], "p32": peaks["p32"], "pdf": peaks["pdf"],

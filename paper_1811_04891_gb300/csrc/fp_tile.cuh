@@ -1310,6 +1310,14 @@ __device__ __forceinline__ void tile_rows_run(TileCtx<n>& X, const NewtonArgs& A
     }
 }
 
+// Listed rows lie in as many elements: a short list is spread over a wave of
+// blocks (the chain of a warp grows with its rows: 100,000 points in 4,096
+// elements, N = 7, 430 us; 490 with at least 16 rows a warp, 570 with 32), a
+// long one takes 32 rows a warp, whose FP64 steps cost the same for any number
+// (a batch of 24 problems 6,040 us with its lists spread over all list blocks,
+// 5,550 us so).
+constexpr int kListSpread = 152;
+
 template <int n, int KIND>
 __global__ void __launch_bounds__(TileLB<KIND>::threads, TileLB<KIND>::blocks) k_newton_tile(NewtonArgs A, BasisTab tab)
 {
@@ -1329,7 +1337,7 @@ __global__ void __launch_bounds__(TileLB<KIND>::threads, TileLB<KIND>::blocks) k
     };
     if (KIND == TILE_FINAL && (int)blockIdx.x < nl) {
         const PairRange L{0, (int64_t)*A.pause_count};
-        for_each_rows(A, L, rows_of(L.s1, nl, 0), false, (int)blockIdx.x, nl, [&](int64_t s0, int64_t s1) {
+        for_each_rows(A, L, rows_of(L.s1, min(nl, kListSpread), 0), false, (int)blockIdx.x, nl, [&](int64_t s0, int64_t s1) {
             tile_rows_run<n, KIND>(X, A, tab, true, pl, fbl, fbc, s0, s1);
         });
         return;
