@@ -65,6 +65,8 @@ template <int n, int KIND>
 static cudaError_t launch_tile(const NewtonArgs& na, const BasisTab& tab, int64_t npairs, int block, unsigned grid,
                                cudaStream_t s)
 {
+    // whole warps, at most the four of the launch bounds: each has its own shared memory
+    if (block < 32 || block > TileLB<KIND>::threads || block % 32 != 0) return cudaErrorInvalidValue;
     const int per = block / 32;
     const cudaError_t err = tile_prepare<n, KIND>();
     if (err != cudaSuccess) return err;
@@ -105,11 +107,24 @@ static int tile_rows(int64_t npairs, int warps)
 
 // Few pairs (a launch of fewer than two blocks per SM at `block` threads):
 // smaller blocks, down to one warp, so that every SM gets work.  The block
-// size changes only the schedule, not any pair's result.
+// size changes only the schedule, not any pair's result.  Blocks stay whole
+// warps (any multiple of 32 may be asked for: 96 goes to 32, not to 48): the
+// tile kernels' warps share no rows and every lane of a warp takes part.
+constexpr int halved_block(int block) { return block / 2 / 32 * 32 < 32 ? 32 : block / 2 / 32 * 32; }
+
+constexpr bool halves_to_whole_warps()
+{
+    for (int b = 32; b <= 1024; b += 32)
+        for (int h = b; h > 32; h = halved_block(h))
+            if (halved_block(h) % 32 != 0 || halved_block(h) < 32 || halved_block(h) >= h) return false;
+    return true;
+}
+static_assert(halves_to_whole_warps(), "spread_block: whole warps only");
+
 static int spread_block(int64_t npairs, int block)
 {
     const int nsm = sm_count();
-    while (block > 32 && (npairs + block - 1) / block < 2 * nsm) block >>= 1;
+    while (block > 32 && (npairs + block - 1) / block < 2 * nsm) block = halved_block(block);
     return block;
 }
 
