@@ -32,7 +32,9 @@ struct ElemBox {
     double bhi[3];      //   ... plus pad
     double he;          // diagonal of the axis box spanned by the element's nodes
     double scale;       // power of two with |x - c| / scale < 1/2 over the nodes (digit form, see fp_tile.cuh)
-    double jscale[2];   // the same for the nodal values of dx/dr and dx/ds, in units of scale
+    float cscale[3];    // the same for each coordinate by itself, in units of scale (at most 1)
+    float jscale[2][3]; // the same for the nodal values of dx/dr and dx/ds, in units of scale
+    float pad_;
     double dev;         // largest distance of a node from its place in the affine frame, |y - xi| (infinity norm);
                         //   infinite where it is not computed
 };

@@ -170,7 +170,9 @@ __global__ void k_hull2(int n, int64_t E, const double* __restrict__ coords, con
         bx.Ai[3] = Ai[2]; bx.Ai[4] = Ai[3];
         bx.Ai[8] = 1.0;
         bx.he = he;
-        bx.scale = bx.jscale[0] = bx.jscale[1] = 1.0;
+        bx.scale = 1.0;
+        for (int a = 0; a < 3; ++a) bx.cscale[a] = bx.jscale[0][a] = bx.jscale[1][a] = 1.0f;
+        bx.pad_ = 0.0f;
         bx.dev = dev;
         boxes[e] = bx;
         nodebox[6 * e + 0] = lo[0]; nodebox[6 * e + 1] = lo[1]; nodebox[6 * e + 2] = 0.0;

@@ -130,7 +130,7 @@ struct FindArgs {
 
 // Tensor-core tile kernels (fp_tile.cuh) of the Newton stage: their orders,
 // the bytes of an element's node digits (0 for other orders) and the kernel
-// that lays them out (also boxes[].scale, jscale and dev).
+// that lays them out (also boxes[].scale, cscale, jscale and dev).
 //
 // The order decides alone, never the number of points, so that every entry
 // point gives a pair the same bits.  Lower orders have too little to contract,

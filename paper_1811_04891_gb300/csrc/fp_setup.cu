@@ -200,7 +200,9 @@ __global__ void k_hull(int n, int64_t E, const double* __restrict__ coords,
         }
         for (int q = 0; q < 9; ++q) bx.Ai[q] = Ai[q];
         bx.he = he;
-        bx.scale = bx.jscale[0] = bx.jscale[1] = 1.0;
+        bx.scale = 1.0;
+        for (int a = 0; a < 3; ++a) bx.cscale[a] = bx.jscale[0][a] = bx.jscale[1][a] = 1.0f;
+        bx.pad_ = 0.0f;
         bx.dev = INFINITY;
         boxes[e] = bx;
         for (int a = 0; a < 3; ++a) {

@@ -13,7 +13,8 @@
 //
 // Exactness.  Both factors are cut into signed 10-bit digits (fixed point:
 // the basis products lie in [-1,1], the node offsets x - c_e are scaled by a
-// power of two per element into [-1/2,1/2]), which FP16 holds exactly.  A
+// power of two per element and coordinate into [-1/2,1/2], so that a thin
+// direction of a stretched element keeps all its bits), which FP16 holds exactly.  A
 // product of two digits has at most 19 bits and the FP32 accumulators add
 // products of equal weight exactly, so the only errors are the last digit's
 // rounding and the orders left out: 5 digits and orders 0..5 give about 2^-50
@@ -380,6 +381,7 @@ struct TileCtx {
     const unsigned char* dig;
     uint32_t heads;                    // rows whose element differs from the row before
     int e;                             // the row's element
+    const ElemBox* bx;
 };
 
 // store one direction's values of this lane's row; the j padding is zero
@@ -421,11 +423,27 @@ __device__ __forceinline__ void contract_out(T* out, T* out2, bool both, const T
     }
 }
 
+// exact FP32 -> FP64 by integer operations: the FP64 pipe takes 16 clocks of
+// an SM for a warp's conversion, these take two
+__device__ __forceinline__ double widen(float f)
+{
+    const uint32_t b = (uint32_t)__float_as_int(f), m = b & 0x7fffffffu;
+    const uint32_t hi = m < 0x00800000u ? 0u : ((m >> 3) + 0x38000000u);
+    return __hiloint2double((int)(hi | (b & 0x80000000u)), m < 0x00800000u ? 0 : (int)(b << 29));
+}
+
+template <typename T>
+__device__ __forceinline__ T scale_of(float f)
+{
+    if constexpr (sizeof(T) == 8) return widen(f);
+    else return f;
+}
+
 // map x(r) in the element's frame and scale, and its Jacobian: T = float (to
 // FP32 accuracy, the mixed form's FP32 phase) or double (FP64 form)
 template <int n, typename T>
 __device__ __forceinline__ void tile_fJ(const TileCtx<n>& X, const BasisTab& tab, uint32_t need, bool jac,
-                                        const T (&r)[3], const T (&js)[2], T (&x)[3], T (&J)[9])
+                                        const T (&r)[3], T (&x)[3], T (&J)[9])
 {
     constexpr bool F64 = sizeof(T) == 8;
     using D = TileDim<n>;
@@ -497,12 +515,15 @@ __device__ __forceinline__ void tile_fJ(const TileCtx<n>& X, const BasisTab& tab
             __syncwarp();
         }
     }
+    // from each coordinate's own scale to the element's
     const T* out = sm + L::OUT + lane;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        x[a] = out[a * kTileRows];
+        const T cs = scale_of<T>(X.bx->cscale[a]);
+        x[a] = out[a * kTileRows] * cs;
 #pragma unroll
-        for (int b = 0; b < 3; ++b) J[3 * a + b] = out[(3 + 3 * b + a) * kTileRows] * (b < 2 ? js[b] : T(1));
+        for (int b = 0; b < 3; ++b)
+            J[3 * a + b] = out[(3 + 3 * b + a) * kTileRows] * (b < 2 ? scale_of<T>(X.bx->jscale[b][a]) : cs);
     }
     __syncwarp();
 }
@@ -567,7 +588,8 @@ __device__ __forceinline__ void tile_f_df(const TileCtx<n>& X, const BasisTab& t
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         const float2 y = sm[L::OUT + a * kTileRows + lane];
-        f[a] = (y.x - xl[a].hi) + (y.y - xl[a].lo);
+        const float cs = X.bx->cscale[a];
+        f[a] = (y.x * cs - xl[a].hi) + (y.y * cs - xl[a].lo);
     }
     __syncwarp();
 }
@@ -761,7 +783,7 @@ __device__ __forceinline__ float inv_norm(const T (&Jd)[9])
 // that the rows of a warp share their evaluations ----
 template <int n>
 __device__ __forceinline__ void tile_solve_f64(const TileCtx<n>& X, const NewtonArgs& A, const BasisTab& tab, bool active,
-                                               const double (&xl)[3], const double (&js)[2], double xmax,
+                                               const double (&xl)[3], double xmax,
                                                double (&r)[3], double& res2, NewtonState& st)
 {
     enum { FIRST, TRIAL, CHORD, REFRESH, DONE };
@@ -778,7 +800,7 @@ __device__ __forceinline__ void tile_solve_f64(const TileCtx<n>& X, const Newton
         const uint32_t wf = __ballot_sync(kFull, state == CHORD);
         if (!(wj | wf)) break;
         double fn[3], Jn[9];
-        tile_fJ<n, double>(X, tab, wj | wf, wj != 0, rn, js, fn, Jn);
+        tile_fJ<n, double>(X, tab, wj | wf, wj != 0, rn, fn, Jn);
         if (state == DONE) continue;
 #pragma unroll
         for (int a = 0; a < 3; ++a) fn[a] -= xl[a];
@@ -896,7 +918,7 @@ __device__ __forceinline__ void tile_solve_f64(const TileCtx<n>& X, const Newton
 // the final steps, with r and J from here.
 template <int n>
 __device__ __forceinline__ bool tile_phase32(const TileCtx<n>& X, const NewtonArgs& A, const BasisTab& tab, bool active,
-                                             const double (&xl)[3], const float (&js)[2], double hes, double (&r)[3],
+                                             const double (&xl)[3], double hes, double (&r)[3],
                                              float (&J)[9], double& res2, int& fate, NewtonState& st)
 {
     enum { FIRST, TRIAL, DONE };
@@ -915,7 +937,7 @@ __device__ __forceinline__ bool tile_phase32(const TileCtx<n>& X, const NewtonAr
         const uint32_t want = __ballot_sync(kFull, state != DONE);
         if (!want) break;
         float fn[3], Jn[9];
-        tile_fJ<n, float>(X, tab, want, true, qn, js, fn, Jn);
+        tile_fJ<n, float>(X, tab, want, true, qn, fn, Jn);
         if (state == DONE) continue;
 #pragma unroll
         for (int a = 0; a < 3; ++a) fn[a] -= (float)xl[a];
@@ -1005,15 +1027,6 @@ __device__ __forceinline__ bool tile_phase32(const TileCtx<n>& X, const NewtonAr
         }
     }
     return final;
-}
-
-// exact FP32 -> FP64 by integer operations: the FP64 pipe takes 16 clocks of
-// an SM for a warp's conversion, these take two
-__device__ __forceinline__ double widen(float f)
-{
-    const uint32_t b = (uint32_t)__float_as_int(f), m = b & 0x7fffffffu;
-    const uint32_t hi = m < 0x00800000u ? 0u : ((m >> 3) + 0x38000000u);
-    return __hiloint2double((int)(hi | (b & 0x80000000u)), m < 0x00800000u ? 0 : (int)(b << 29));
 }
 
 // ---- mixed form: the final steps on compensated residuals (see solve_mixed)
@@ -1215,6 +1228,7 @@ __device__ __forceinline__ void tile_rows_run(TileCtx<n>& X, const NewtonArgs& A
     X.e = e;
     X.heads = __ballot_sync(kFull, lane == 0 || e != eprev);
     const ElemBox& bx = A.boxes[e];
+    X.bx = &bx;
     const double xs[3] = {A.pts[p], A.pts[A.P + p], A.pts[2 * A.P + p]};
     const double xc[3] = {xs[0] - bx.c[0], xs[1] - bx.c[1], xs[2] - bx.c[2]};
     const double scale = bx.scale, inv = 1.0 / scale;     // a power of two: exact
@@ -1251,8 +1265,7 @@ __device__ __forceinline__ void tile_rows_run(TileCtx<n>& X, const NewtonArgs& A
     if constexpr (KIND == TILE_FP64) {
         if (scans) tile_seed_nearest<n, double>(A.coords, A.E, scans, e, xs, tab.xi, r);
         const double xmax = fmax(fabs(xs[0]), fmax(fabs(xs[1]), fabs(xs[2]))) * inv;
-        const double js[2] = {bx.jscale[0], bx.jscale[1]};
-        tile_solve_f64<n>(X, A, tab, active, xl, js, xmax, r, res2, st);
+        tile_solve_f64<n>(X, A, tab, active, xl, xmax, r, res2, st);
     } else {
         if (KIND != TILE_FINAL && scans) {
             const float x32[3] = {(float)xc[0], (float)xc[1], (float)xc[2]};
@@ -1261,8 +1274,7 @@ __device__ __forceinline__ void tile_rows_run(TileCtx<n>& X, const NewtonArgs& A
             r[0] = rs[0]; r[1] = rs[1]; r[2] = rs[2];
         }
         if (KIND != TILE_FINAL || listed) {
-            const float js[2] = {(float)bx.jscale[0], (float)bx.jscale[1]};
-            const bool f = tile_phase32<n>(X, A, tab, active && !final, xl, js, hes, r, J, res2, fate, st);
+            const bool f = tile_phase32<n>(X, A, tab, active && !final, xl, hes, r, J, res2, fate, st);
             final = final || f;
         }
         if (KIND == TILE_MIXED || (KIND == TILE_FINAL && listed)) tile_final<n, true>(X, A, tab, final, xl, hes, r, J, res2, fate);
@@ -1364,6 +1376,14 @@ struct DigitsSm {
     static constexpr int bytes = V * (int)(sizeof(double) + (MIXED ? 2 : 1) * sizeof(TJ)) + n * n * (int)sizeof(TJ);
 };
 
+// exponent of a magnitude, so that v < 2^(exponent - 1022); integer maxima of
+// these take one instruction a warp, FP64 ones a pass over its pipe each
+__device__ __forceinline__ int expo(double v) { return (__double2hiint(v) >> 20) & 0x7ff; }
+__device__ __forceinline__ int expo(float v) { const int e = (__float_as_int(v) >> 23) & 0xff; return e ? e + 896 : 0; }
+
+// k with 2^k > 2 |v| where expo(v) <= e, at least `least` (that also for e = 0)
+__device__ __forceinline__ int scale_exp(int e, int least) { return min(1000, max(e > 0 ? e - 1021 : least, least)); }
+
 template <int n, bool MIXED>
 __global__ void __launch_bounds__(128) k_digits(int64_t E, const double* __restrict__ coords, ElemBox* boxes,
                                                 unsigned char* __restrict__ dig, BasisTab tab)
@@ -1378,7 +1398,7 @@ __global__ void __launch_bounds__(128) k_digits(int64_t E, const double* __restr
     TJ* W = reinterpret_cast<TJ*>(V + L::V);
     TJ* Vj = MIXED ? W + L::V : reinterpret_cast<TJ*>(V);
     TJ* der = W + (MIXED ? 2 : 1) * L::V;                 // der[i n + m] = h_m'(xi_i)
-    __shared__ double red[8];
+    __shared__ int4 red[4];
     const int64_t e = blockIdx.x;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (threadIdx.x < n) {
@@ -1392,7 +1412,21 @@ __global__ void __launch_bounds__(128) k_digits(int64_t E, const double* __restr
 #pragma unroll
         for (int m = 0; m < n; ++m) der[threadIdx.x * n + m] = d[m];
     }
-    double mx = 0.0, dev = 0.0;
+    // the largest of four values over the block, none negative
+    auto block_max = [&](int4 v) {
+        v = make_int4(__reduce_max_sync(kFull, v.x), __reduce_max_sync(kFull, v.y), __reduce_max_sync(kFull, v.z),
+                      __reduce_max_sync(kFull, v.w));
+        __syncthreads();
+        if (lane == 0) red[warp] = v;
+        __syncthreads();
+#pragma unroll
+        for (int w = 0; w < 4; ++w) {
+            const int4 o = red[w];
+            v = make_int4(max(v.x, o.x), max(v.y, o.y), max(v.z, o.z), max(v.w, o.w));
+        }
+        return v;
+    };
+    int4 most = make_int4(0, 0, 0, 0);                    // exponents per coordinate; the deviation's bits
     {
         double c[3];
         float Ai[9];
@@ -1408,38 +1442,35 @@ __global__ void __launch_bounds__(128) k_digits(int64_t E, const double* __restr
             for (int a = 0; a < 3; ++a) {
                 v[a] = coords[((int64_t)a * E + e) * n3 + q] - c[a];
                 V[a * n * PL + at] = v[a];
-                mx = fmax(mx, fabs(v[a]));
                 vf[a] = (float)v[a];
             }
+            most = make_int4(max(most.x, expo(v[0])), max(most.y, expo(v[1])), max(most.z, expo(v[2])), most.w);
 #pragma unroll
             for (int a = 0; a < 3; ++a)
-                dev = fmax(dev, (double)fabsf(Ai[3 * a] * vf[0] + Ai[3 * a + 1] * vf[1] + Ai[3 * a + 2] * vf[2] -
-                                              tab.xif[id[a]]));
+                most.w = max(most.w, __float_as_int(fabsf(Ai[3 * a] * vf[0] + Ai[3 * a + 1] * vf[1] + Ai[3 * a + 2] * vf[2] -
+                                                         tab.xif[id[a]])));
         }
     }
-    auto reduce = [&](double v, int at) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(kFull, v, o));
-        if (lane == 0) red[at + warp] = v;
-        __syncthreads();
-        return fmax(fmax(red[at], red[at + 1]), fmax(red[at + 2], red[at + 3]));
-    };
-    mx = reduce(mx, 0);
-    dev = reduce(dev, 4);
-    const int ex = mx > 0.0 ? ilogb(mx) + 2 : 0;          // |x - c| / scale < 1/2
-    const double inv = ldexp(1.0, -ex);
+    most = block_max(most);
+    const float dev = __int_as_float(most.w);
+    const int all = max(most.x, max(most.y, most.z)), ex = all > 0 ? scale_exp(all, -1000) : 0;
+    // not below 2^-100 of the largest: within FP32's range
+    const int3 ea = make_int3(scale_exp(most.x, ex - 100), scale_exp(most.y, ex - 100), scale_exp(most.z, ex - 100));
     for (int i = threadIdx.x; i < L::V; i += 128) {       // (the padding too: never read back)
-        const double v = V[i] * inv;
+        const int a = i / (n * PL);
+        const double v = V[i] * ldexp(1.0, -(a == 0 ? ea.x : a == 1 ? ea.y : ea.z));
         V[i] = v;
         if (MIXED) Vj[i] = (TJ)v;
     }
     __syncthreads();
-    auto frags = [&](auto* val, auto ji, unsigned char* out, auto digits) {
+    // digits of the values val[], each coordinate divided by its power of two
+    auto frags = [&](auto* val, int3 sa, unsigned char* out, auto digits) {
         constexpr int SD = decltype(digits)::value;
         using TV = std::conditional_t<SD == 5, double, float>;
         for (int f = warp; f < D::KC * D::NT; f += 4) {
             const int kc = f / D::NT, t = f % D::NT, g = lane >> 2, q = lane & 3;
             const int col = 8 * t + g;                    // column a n + k is plane a n + k
+            const TV ji = ldexp(TV(1), -(col < n ? sa.x : col < 2 * n ? sa.y : sa.z));
             uint32_t b[5][2];
 #pragma unroll
             for (int hf = 0; hf < 2; ++hf) {
@@ -1450,8 +1481,7 @@ __global__ void __launch_bounds__(128) k_digits(int64_t E, const double* __restr
                     v[u] = kap < D::n2 && col < 3 * n ? (TV)val[col * PL + kap] : TV(0);
                 }
                 uint32_t d[SD];
-                if constexpr (SD == 5) digits2(v[0], (double)ji, v[1], (double)ji, d);
-                else digits2(v[0], ji, v[1], ji, d);
+                digits2(v[0], ji, v[1], ji, d);
 #pragma unroll
                 for (int s = 0; s < SD; ++s) b[s][hf] = d[s];
             }
@@ -1466,12 +1496,11 @@ __global__ void __launch_bounds__(128) k_digits(int64_t E, const double* __restr
         }
     };
     unsigned char* out = dig + e * TB::v;
-    frags(V, 1.0, out, std::integral_constant<int, 5>());
-    // dx/dr and dx/ds, each with its own power of two
-    double js[2];
+    frags(V, make_int3(0, 0, 0), out, std::integral_constant<int, 5>());
+    // dx/dr and dx/ds, each coordinate with its own power of two
 #pragma unroll 1
     for (int m = 0; m < 2; ++m) {
-        double wm = 0.0;
+        most = make_int4(0, 0, 0, 0);
         for (int i = threadIdx.x; i < 3 * n3; i += 128) {
             const int c = i / (n * n), q = i % (n * n), at = m == 0 ? q % n : q / n, st = m == 0 ? 1 : n;
             const TJ* v = Vj + c * PL + q - at * st;
@@ -1479,18 +1508,27 @@ __global__ void __launch_bounds__(128) k_digits(int64_t E, const double* __restr
 #pragma unroll
             for (int u = 0; u < n; ++u) w += der[at * n + u] * v[u * st];
             W[c * PL + q] = w;
-            wm = fmax(wm, (double)fabs(w));
+            const int x = expo(w);
+            if (i < n3) most.x = max(most.x, x);
+            else if (i < 2 * n3) most.y = max(most.y, x);
+            else most.z = max(most.z, x);
         }
-        wm = reduce(wm, 4 * m);
-        js[m] = ldexp(1.0, wm > 0.0 ? ilogb(wm) + 2 : 0);
-        frags(W, (TJ)(1.0 / js[m]), out + TB::jac + m * TB::one, std::integral_constant<int, TB::SJ>());
+        most = block_max(most);
+        const int3 sa = make_int3(scale_exp(most.x, -100), scale_exp(most.y, -100), scale_exp(most.z, -100));
+        frags(W, sa, out + TB::jac + m * TB::one, std::integral_constant<int, TB::SJ>());
+        if (threadIdx.x == 0) {
+            boxes[e].jscale[m][0] = ldexpf(1.0f, sa.x + ea.x - ex);
+            boxes[e].jscale[m][1] = ldexpf(1.0f, sa.y + ea.y - ex);
+            boxes[e].jscale[m][2] = ldexpf(1.0f, sa.z + ea.z - ex);
+        }
         __syncthreads();                                  // W is rewritten
     }
     if (threadIdx.x == 0) {
         boxes[e].scale = ldexp(1.0, ex);
         boxes[e].dev = dev;
-        boxes[e].jscale[0] = js[0];
-        boxes[e].jscale[1] = js[1];
+        boxes[e].cscale[0] = ldexpf(1.0f, ea.x - ex);
+        boxes[e].cscale[1] = ldexpf(1.0f, ea.y - ex);
+        boxes[e].cscale[2] = ldexpf(1.0f, ea.z - ex);
     }
 }
 
