@@ -15,14 +15,22 @@
 // the basis products lie in [-1,1], the node offsets x - c_e are scaled by a
 // power of two per element and coordinate into [-1/2,1/2], so that a thin
 // direction of a stretched element keeps all its bits), which FP16 holds exactly.  A
-// product of two digits has at most 19 bits and the FP32 accumulators add
-// products of equal weight exactly, so the only errors are the last digit's
-// rounding and the orders left out: 5 digits and orders 0..5 give about 2^-50
-// of the element's size (FP64 form; global FP64 coordinates carry 2^-53 of
-// |x|), orders 0..4 about 2^-48 (the mixed form's compensated residuals), 3
-// digits and orders 0..2 about 2^-27 (its FP32 phase).  A row's sums do not
-// depend on the other rows, so a pair's result does not depend on which
-// pairs share its warp, on the block size, or on the entry point.
+// product of two digits has at most 19 bits, and the FP32 accumulators add
+// products of equal weight exactly as long as a sum stays below 2^24.  Orders
+// 0 and 1 do (one factor's first digits add up to at most 512 times the
+// Lebesgue constant squared, 100 products of 2^17 the other way); for the
+// others, sums of n^2 products of digits of either sign, it is a matter of
+// odds: 2^23 is the largest seen over 200 random points for N = 3 to 9, 2^24
+// is more than 10 standard deviations.  What is left is the last digit's
+// rounding and the orders left out.  FP64 form: 6 digits and orders 0..5,
+// 2^-58 of the element's size, below an FP64 sum's own rounding (error of x(r)
+// against extended precision, relative to half the element's width, N = 7,
+// width 0.1: 2e-16 rms; by FP64 sum factorisation 3e-16 for coordinates
+// around zero, 3e-15 around 0.5; with 5 digits 3e-15).  Mixed form: 5 digits
+// and orders 0..4, about 2^-48 (compensated residuals), 3 digits and orders
+// 0..2, about 2^-27 (its FP32 phase).  A row's sums do not depend on the other
+// rows, so a pair's result does not depend on which pairs share its warp, on
+// the block size, or on the entry point.
 //
 // Layout.  A warp takes `rows` consecutive element-sorted pairs, at most 32;
 // lane l keeps pair l's Newton state and evaluates its Lagrange bases.  The
@@ -30,7 +38,10 @@
 // mma.m16n8k16 fragments and loop over the elements among the pairs (rows of
 // other elements masked to zero).  The nodes' digits are laid out once per
 // mesh in fragment order, so a fragment is one coalesced load; with three
-// digits the next one is fetched while the current one is multiplied.  Tiles
+// digits the next one is fetched while the current one is multiplied.  The
+// FP64 form takes dx/dr and dx/ds from the same node digits with h_i' h_j and
+// h_i h_j' on the left: a third of the memory, set-up time and L2 traffic of
+// digits of the derivatives for two more left factors.  Tiles
 // of 128 pairs per tcgen05.mma would leave most rows empty (1 to 300 pairs
 // per element are typical), and the 16-row form is already bound by building
 // the digits, by the latency of its chain (16 warps an SM) and by issue
@@ -64,28 +75,29 @@ struct TileDim {
 };
 
 // Shared memory of one warp: the basis values h_i(r), h_j(s), h_k(t), h_k'(t)
-// of its 32 rows, the left factor's digits of one 16-row tile (fragment
-// order), the columns c of one tile, and the results (x, dx/dr, dx/ds, dx/dt
-// in three coordinates).  Row strides of 34 and 18 eight-byte values (36 and
+// (FP64 form: also h_i'(r) and h_j'(s)) of its 32 rows, the left factor's digits of one 16-row tile (fragment
+// order), the columns c of one tile, and the results (x, dx/dr, dx/ds in three
+// coordinates; dx/dt takes the place of a row's h_k'(t)).  Row strides of 34 and 18 eight-byte values (36 and
 // 20 floats) put the fragment accesses of a half-warp into distinct banks.
 template <typename T> struct TileStride {
     static constexpr int H = sizeof(T) == 4 ? 36 : 34, C = sizeof(T) == 4 ? 20 : 18;
 };
 
-template <int n, typename T, int S, int NH, int NO>      // NH: 3 or 4 basis arrays, NO: result quantities
+template <int n, typename T, int S, int NH, int NO>      // NH: 3, 4 or 6 basis arrays, NO: result quantities
 struct TileSm {
     using D = TileDim<n>;
-    static constexpr int HR = 0, HS = HR + n * TileStride<T>::H, HT = HS + D::JP * TileStride<T>::H,
-                         DT = HT + n * TileStride<T>::H, C = HT + (NH - 2) * n * TileStride<T>::H,
-                         OUT = C + 3 * n * TileStride<T>::C, VALS = OUT + 3 * NO * kTileRows;
+    static constexpr int H = TileStride<T>::H;
+    static constexpr int HR = 0, HS = HR + n * H, DR = HS + D::JP * H, DS = DR + n * H,
+                         HT = NH == 6 ? DS + D::JP * H : DR, DT = HT + n * H, C = NH == 3 ? DT : DT + n * H,
+                         OUT = C + 3 * n * TileStride<T>::C, VALS = OUT + 3 * NO * kTileRows;   // (dx/dt: in DT)
     // the digits start on a 16-byte boundary
     static constexpr int DIG = (int)((VALS * sizeof(T) + 15) / 16 * 16);
     static constexpr int BYTES = DIG + (S > 0 ? D::KC * S * 512 : 0);
 };
 
-template <int n> using Sm32 = TileSm<n, float, 3, 4, 4>;    // FP32 phase
+template <int n> using Sm32 = TileSm<n, float, 3, 4, 3>;    // FP32 phase
 template <int n> using SmDf = TileSm<n, float2, 0, 3, 1>;   // compensated residual: digits stay in registers
-template <int n> using Sm64 = TileSm<n, double, 5, 4, 4>;   // FP64 form
+template <int n> using Sm64 = TileSm<n, double, 0, 6, 3>;   // FP64 form: the same
 
 __device__ __forceinline__ void mma_16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
 {
@@ -149,45 +161,62 @@ __device__ __forceinline__ void digits2(float2 a0, float2 b0, float2 a1, float2 
     o[4] = pack_h2(digit<49>(v));
 }
 
-// FP64 products, rounded to 2^-49 by one fused multiply-add (12 + a b has
-// its last bit there); the digits are bit fields of the sum
-__device__ __forceinline__ uint64_t fix49(double a, double b)
+// FP64 form: a basis value in [-1,1] as x 2^-30 + y 2^-60, |y| <= 2^29: the low
+// words of the sums with 1.5 2^22 and 1.5 2^-8 (last bits 2^-30 and 2^-60; the
+// difference between them is exact)
+__device__ __forceinline__ int2 fix60(double h)
 {
-    // 512 at every digit's weight: the fields hold digit + 512
-    constexpr uint64_t bias = (512ull << 40) | (512ull << 30) | (512ull << 20) | (512ull << 10) | 512ull;
-    return (uint64_t)__double_as_longlong(fma(a, b, 12.0)) - 0x4028000000000000ull + bias;
+    const double p = h + 0x1.8p22, q = h + ((0x1.8p22 + 0x1.8p-8) - p);
+    return make_int2(__double2loint(p), __double2loint(q));
 }
 
-__device__ __forceinline__ void digits2(double a0, double b0, double a1, double b1, uint32_t (&o)[5])
+// the product of two of them in units of 2^-60 (y y' left out), by integer
+// multiply-adds: the FP64 pipe, with 3 operations a product, was what bounded
+// the kernel (2.0e6 points, N = 7, whole find and evaluation: 26.1 ms).  The
+// bias makes digit s the bits 51 - 10 s and up, plus 512, rounded to 2^-59.
+__device__ __forceinline__ uint64_t product60(int2 a, int2 b)
 {
-    const uint64_t u = fix49(a0, b0), w = fix49(a1, b1);
+    constexpr int64_t bias = 512ll * ((1ll << 51) + (1ll << 41) + (1ll << 31) + (1ll << 21) + (1ll << 11) + (1ll << 1)) + 1;
+    const int64_t low = (int64_t)a.x * b.y + ((int64_t)a.y * b.x + (1 << 29));
+    return (uint64_t)(((int64_t)a.x * b.x + bias) + (low >> 30));
+}
+
+// three digits of two products, as FP16 pairs: f is the FP16 number 1024 + f
+// (bits 0x6400 + f) minus 1536; the first digit of all reaches 512 (11 bits)
+template <bool FIRST>
+__device__ __forceinline__ void fields3(uint32_t u, uint32_t w, uint32_t* o)
+{
     const __half2 off = __floats2half2_rn(1536.0f, 1536.0f);
-    // a field f as the FP16 number 1024 + f (bits 0x6400 + f), minus 1536
 #pragma unroll
-    for (int s = 0; s < 5; ++s) {
-        const uint32_t x = (uint32_t)(u >> (10 * (4 - s))), y = (uint32_t)(w >> (10 * (4 - s)));
-        const uint32_t m = s == 0 ? 0x07ff07ffu : 0x03ff03ffu;
-        uint32_t v = __byte_perm(x, y, 0x5410) & m;
-        v = s == 0 ? v + 0x64006400u : v | 0x64006400u;
+    for (int s = 0; s < 3; ++s) {
+        uint32_t v = __byte_perm(u >> (10 * (2 - s)), w >> (10 * (2 - s)), 0x5410);
+        v = FIRST && s == 0 ? (v & 0x07ff07ffu) + 0x64006400u : (v & 0x03ff03ffu) | 0x64006400u;
         o[s] = h2bits(__hsub2(*reinterpret_cast<__half2*>(&v), off));
     }
 }
 
+// 6 digits
+__device__ __forceinline__ void digits2(int2 a0, int2 b0, int2 a1, int2 b1, uint32_t (&o)[6])
+{
+    const uint64_t u = product60(a0, b0), w = product60(a1, b1);
+    fields3<true>((uint32_t)(u >> 31), (uint32_t)(w >> 31), o);
+    fields3<false>((uint32_t)(u >> 1), (uint32_t)(w >> 1), o + 3);
+}
+
 // ---- the element's nodes as digits, in B-fragment order ----
-// per element: the nodes x (KC x NT fragments), then the nodal values of
-// dx/dr and dx/ds (the derivative of the interpolant is the interpolant of
-// its nodal values), so that x, dx/dr and dx/ds share the left factor
-// h_i h_j.  A fragment of 5 digits: 32 lanes x (digits 0,1), 32 lanes x
-// (digits 2,3), 32 lanes x digit 4; of 3 digits (derivatives in the mixed
-// form): 32 lanes x (digits 0,1), 32 lanes x digit 2.  A lane's digit is two
-// registers of two FP16 values.
+// per element: the nodes x (KC x NT fragments; 6 digits in the FP64 form, 5 in
+// the mixed form) and, mixed form, the nodal values of dx/dr and dx/ds in 3
+// digits (the derivative of the interpolant is the interpolant of its nodal
+// values), so that x, dx/dr and dx/ds share the left factor h_i h_j.  A
+// fragment: 32 lanes x (digits 0,1), 32 lanes x (digits 2,3), ..., an odd last
+// digit by itself.  A lane's digit is two registers of two FP16 values.
 template <int S> struct FragBytes { static constexpr int v = 32 * 8 * S; };
 
 template <int n, bool MIXED>
 struct TileBytes {
-    static constexpr int SJ = MIXED ? 3 : 5;             // digits of the derivatives
+    static constexpr int SX = MIXED ? 5 : 6;             // digits of the nodes
     static constexpr int64_t frags = (int64_t)TileDim<n>::KC * TileDim<n>::NT;
-    static constexpr int64_t jac = frags * FragBytes<5>::v, one = frags * FragBytes<SJ>::v, v = jac + 2 * one;
+    static constexpr int64_t jac = frags * FragBytes<SX>::v, one = MIXED ? frags * FragBytes<3>::v : 0, v = jac + 2 * one;
 };
 
 // which rows of a 16-row tile start a new element
@@ -215,56 +244,44 @@ __device__ __forceinline__ void tile_left(const T* hi, const T* hj, int kc, int 
     }
 }
 
-// the right factor's fragments of one k16 step: S digits of NT tiles (sb >= S
-// digits stored)
-template <int n, int S>
+// a fragment of the right factor: S digits of one 8-column tile, of sb stored
+template <int S>
 struct RightFrag {
-    uint32_t b[TileDim<n>::NT][S][2];
-    __device__ __forceinline__ void load(const unsigned char* __restrict__ base, int sb)
+    uint32_t b[S][2];
+    __device__ __forceinline__ void load(const unsigned char* __restrict__ F, int sb)
     {
         const int lane = threadIdx.x & 31;
 #pragma unroll
-        for (int t = 0; t < TileDim<n>::NT; ++t) {
-            const unsigned char* F = base + t * (S == 5 ? FragBytes<5>::v : FragBytes<1>::v * sb);
-            const uint4 b01 = __ldg(reinterpret_cast<const uint4*>(F) + lane);
-            b[t][0][0] = b01.x; b[t][0][1] = b01.y; b[t][1][0] = b01.z; b[t][1][1] = b01.w;
-            if constexpr (S == 3) {
-                const uint2 b2 = __ldg(reinterpret_cast<const uint2*>(F + 512) + (sb == 5 ? 2 * lane : lane));
-                b[t][2][0] = b2.x; b[t][2][1] = b2.y;
-            } else {
-                const uint4 b23 = __ldg(reinterpret_cast<const uint4*>(F + 512) + lane);
-                const uint2 b4 = __ldg(reinterpret_cast<const uint2*>(F + 1024) + lane);
-                b[t][2][0] = b23.x; b[t][2][1] = b23.y; b[t][3][0] = b23.z; b[t][3][1] = b23.w;
-                b[t][4][0] = b4.x; b[t][4][1] = b4.y;
-            }
+        for (int u = 0; u + 1 < S; u += 2) {
+            const uint4 v = __ldg(reinterpret_cast<const uint4*>(F + 256 * u) + lane);
+            b[u][0] = v.x; b[u][1] = v.y; b[u + 1][0] = v.z; b[u + 1][1] = v.w;
         }
+        if constexpr (S % 2 == 1) {
+            const uint2 v = __ldg(reinterpret_cast<const uint2*>(F + 256 * (S - 1)) + (sb > S ? 2 * lane : lane));
+            b[S - 1][0] = v.x; b[S - 1][1] = v.y;
+        }
+    }
+    __device__ __forceinline__ void store(unsigned char* F) const
+    {
+        const int lane = threadIdx.x & 31;
+#pragma unroll
+        for (int u = 0; u + 1 < S; u += 2)
+            reinterpret_cast<uint4*>(F + 256 * u)[lane] = make_uint4(b[u][0], b[u][1], b[u + 1][0], b[u + 1][1]);
+        if constexpr (S % 2 == 1) reinterpret_cast<uint2*>(F + 256 * (S - 1))[lane] = make_uint2(b[S - 1][0], b[S - 1][1]);
     }
 };
 
-// acc[o][t] += the order-o products of S left and S right digits; FINE adds
-// order 5 to the order-4 sums (left digits scaled by 2^-10)
-template <int n, int S, int O, bool FINE>
-__device__ __forceinline__ void mma_digits(const uint32_t (&a)[S][4], const RightFrag<n, S>& R,
+// acc[o][t] += the order-o products of S left digits and the S right digits of
+// tile t
+template <int n, int S, int O>
+__device__ __forceinline__ void mma_digits(const uint32_t (&a)[S][4], const RightFrag<S>& R, int t,
                                            float (&acc)[O][TileDim<n>::NT][4])
 {
 #pragma unroll
-    for (int t = 0; t < TileDim<n>::NT; ++t)
+    for (int u = 0; u < S; ++u)
 #pragma unroll
-        for (int u = 0; u < S; ++u)
-#pragma unroll
-            for (int s = 0; s < S; ++s)
-                if (s + u < O) mma_16816(acc[s + u][t], a[s], R.b[t][u][0], R.b[t][u][1]);
-    if constexpr (FINE) {
-        const __half2 sc = __floats2half2_rn(pow2<-10>(), pow2<-10>());
-#pragma unroll
-        for (int s = 1; s < S; ++s) {
-            uint32_t as[4];
-#pragma unroll
-            for (int v = 0; v < 4; ++v) as[v] = h2bits(__hmul2(*reinterpret_cast<const __half2*>(&a[s][v]), sc));
-#pragma unroll
-            for (int t = 0; t < TileDim<n>::NT; ++t) mma_16816(acc[O - 1][t], as, R.b[t][S - s][0], R.b[t][S - s][1]);
-        }
-    }
+        for (int s = 0; s < S; ++s)
+            if (s + u < O) mma_16816(acc[s + u][t], a[s], R.b[u][0], R.b[u][1]);
 }
 
 // acc = the digit products of a 16-row tile over all k16 steps.  left(kc, a)
@@ -273,7 +290,7 @@ __device__ __forceinline__ void mma_digits(const uint32_t (&a)[S][4], const Righ
 // fetched while the current ones are multiplied (three digits: they fit the
 // registers).  Several: each element's rows in turn, the others masked to
 // zero.
-template <int n, int S, int O, bool FINE, typename Left>
+template <int n, int S, int O, typename Left>
 __device__ __forceinline__ void tile_gemm(Left&& left, const unsigned char* __restrict__ base, int sb, int64_t ebytes,
                                           uint32_t heads, uint32_t need, int e, int mt,
                                           float (&acc)[O][TileDim<n>::NT][4])
@@ -297,18 +314,27 @@ __device__ __forceinline__ void tile_gemm(Left&& left, const unsigned char* __re
     }
     if (!hs) return;
     auto frag = [&](int h, int kc) { return base + (int64_t)__shfl_sync(kFull, e, 16 * mt + h) * ebytes + kc * step; };
-    RightFrag<n, S> next;
-    if (S == 3) next.load(frag(__ffs(hs) - 1, 0), sb);
-    if (S == 3 && heads == 1u) {
+    RightFrag<S> next[S == 3 ? D::NT : 1];
+    auto fetch = [&](const unsigned char* F) {
+#pragma unroll
+        for (int t = 0; t < D::NT; ++t) next[t].load(F + t * FragBytes<1>::v * sb, sb);
+    };
+    if constexpr (S == 3) {
+        fetch(frag(__ffs(hs) - 1, 0));
+        if (heads == 1u) {
 #pragma unroll 1
-        for (int kc = 0; kc < D::KC; ++kc) {
-            const RightFrag<n, S> R = next;
-            if (kc + 1 < D::KC) next.load(frag(0, kc + 1), sb);
-            uint32_t a[S][4];
-            left(kc, a);
-            mma_digits<n, S, O, FINE>(a, R, acc);
+            for (int kc = 0; kc < D::KC; ++kc) {
+                RightFrag<S> R[D::NT];
+#pragma unroll
+                for (int t = 0; t < D::NT; ++t) R[t] = next[t];
+                if (kc + 1 < D::KC) fetch(frag(0, kc + 1));
+                uint32_t a[S][4];
+                left(kc, a);
+#pragma unroll
+                for (int t = 0; t < D::NT; ++t) mma_digits<n, S, O>(a, R[t], t, acc);
+            }
+            return;
         }
-        return;
     }
 #pragma unroll 1
     for (int kc = 0; kc < D::KC; ++kc) {
@@ -319,13 +345,6 @@ __device__ __forceinline__ void tile_gemm(Left&& left, const unsigned char* __re
         while (hm) {
             const int h = __ffs(hm) - 1;
             hm &= hm - 1;
-            RightFrag<n, S> R;
-            if constexpr (S == 3) {
-                R = next;
-                if (hm || kc + 1 < D::KC) next.load(frag(__ffs(hm ? hm : hs) - 1, hm ? kc : kc + 1), sb);
-            } else {
-                R.load(frag(h, kc), sb);
-            }
             const uint32_t after = heads & ~((2u << h) - 1u);
             const int nx = after ? __ffs(after) - 1 : 16;
             uint32_t am[S][4];
@@ -337,7 +356,22 @@ __device__ __forceinline__ void tile_gemm(Left&& left, const unsigned char* __re
                 am[s][2] = a[s][2] & m0;
                 am[s][3] = a[s][3] & m1;
             }
-            mma_digits<n, S, O, FINE>(am, R, acc);
+            if constexpr (S == 3) {
+                RightFrag<S> R[D::NT];
+#pragma unroll
+                for (int t = 0; t < D::NT; ++t) R[t] = next[t];
+                if (hm || kc + 1 < D::KC) fetch(frag(__ffs(hm ? hm : hs) - 1, hm ? kc : kc + 1));
+#pragma unroll
+                for (int t = 0; t < D::NT; ++t) mma_digits<n, S, O>(am, R[t], t, acc);
+            } else {
+                const unsigned char* F = frag(h, kc);
+#pragma unroll
+                for (int t = 0; t < D::NT; ++t) {
+                    RightFrag<S> R;
+                    R.load(F + t * FragBytes<1>::v * sb, sb);
+                    mma_digits<n, S, O>(am, R, t, acc);
+                }
+            }
         }
     }
 }
@@ -363,15 +397,17 @@ __device__ __forceinline__ df2 column_df(float2 a0, float2 a1, float2 a2, float2
     return {__fmul2_rn(s, f2(pow2<-18>())), __fmul2_rn(lo, f2(pow2<-18>()))};
 }
 
-// FP64: the sums are whole numbers; together with the rounded last order they
-// are one 52-bit whole number in units of 2^-49, converted by the exponent
-// trick (1.5 * 2^52 + v) - 1.5 * 2^52
-__device__ __forceinline__ double column_f64(float a0, float a1, float a2, float a3, float a4)
+// FP64, in units of 2^-58: the sums are whole numbers; orders 0 and 1 make one
+// in units of 2^-28, the others (order 5 rounded) one in units of 2^-58, and
+// their bits in 1.5 2^82 and 1.5 2^52 give the two as FP64 numbers, added with
+// one rounding
+__device__ __forceinline__ double column_f64(float a0, float a1, float a2, float a3, float a4, float a5)
 {
     const int64_t hi = (int64_t)__float2int_rn(a0) * 1024 + __float2int_rn(a1);
-    const int64_t lo = (int64_t)__float2int_rn(a2) * 1024 + __float2int_rn(a3);
-    const int64_t v = hi * (1 << 21) + lo * 2 + __float2int_rn(a4 * pow2<-9>());
-    return __longlong_as_double(v + 0x4338000000000000ll) - 6755399441055744.0;
+    const int64_t lo = ((int64_t)__float2int_rn(a2) * 1024 + __float2int_rn(a3)) * 1024 + __float2int_rn(a4) +
+                       __float2int_rn(a5 * pow2<-10>());
+    const double H = __longlong_as_double(hi + 0x4518000000000000ll), W = __longlong_as_double(lo + 0x4338000000000000ll);
+    return (H - (0x1.8p82 + 0x1.8p52)) + W;
 }
 
 // ---- collective evaluations: lane l holds row l ----
@@ -395,11 +431,11 @@ __device__ __forceinline__ void store_dir(T* p, bool pad, const T (&h)[n])
         for (int i = n; i < TileDim<n>::JP; ++i) p[i * TileStride<T>::H] = T{};
 }
 
-// sum_k w_k c[a n + k] of a 16-row tile, times u, into the results: a = 0
+// sum_k w_k c[a n + k] of a 16-row tile into the results: a = 0
 // (lanes < 16) and 1 (lanes >= 16) in one pass, then a = 2; with `both` also
-// the sums with the second weights, into out2
+// the sums with the second weights, over these
 template <int n, typename T>
-__device__ __forceinline__ void contract_out(T* out, T* out2, bool both, const T* c, const T* w, const T* w2, T u)
+__device__ __forceinline__ void contract_out(T* out, bool both, const T* c, const T* w, T* w2)
 {
     constexpr int PS = TileStride<T>::C, HS = TileStride<T>::H;
     const int lane = threadIdx.x & 31, row = lane & 15, a01 = lane >> 4;
@@ -415,11 +451,12 @@ __device__ __forceinline__ void contract_out(T* out, T* out2, bool both, const T
             t2 = fma(vk, ck2, t2);
         }
     }
-    out[a01 * kTileRows + row] = s * u;
-    if (lane < 16) out[2 * kTileRows + row] = s2 * u;
+    out[a01 * kTileRows + row] = s;
+    if (lane < 16) out[2 * kTileRows + row] = s2;
     if (both) {
-        out2[a01 * kTileRows + row] = t * u;
-        if (lane < 16) out2[2 * kTileRows + row] = t2 * u;
+        __syncwarp();                                     // both of a row's lanes have read w2
+        w2[a01 * HS + row] = t;
+        if (lane < 16) w2[2 * HS + row] = t2;
     }
 }
 
@@ -432,12 +469,17 @@ __device__ __forceinline__ double widen(float f)
     return __hiloint2double((int)(hi | (b & 0x80000000u)), m < 0x00800000u ? 0 : (int)(b << 29));
 }
 
-template <typename T>
+// a power of two f times 2^e (FP64: e goes into the exponent)
+template <typename T, int e = 0>
 __device__ __forceinline__ T scale_of(float f)
 {
-    if constexpr (sizeof(T) == 8) return widen(f);
-    else return f;
+    if constexpr (sizeof(T) == 8) return __hiloint2double((__float_as_int(f) >> 3) + 0x38000000 + e * 0x100000, 0);
+    else return f * pow2<e>();
 }
+
+// |h_i'| <= N^2 <= 2^kDerivExp on the reference interval (Markov's inequality
+// for |h_i| <= 1): the derivatives' factor in the FP64 form
+template <int n> constexpr int kDerivExp = n <= 4 ? 4 : n <= 5 ? 4 : n <= 6 ? 5 : n <= 9 ? 6 : 7;
 
 // map x(r) in the element's frame and scale, and its Jacobian: T = float (to
 // FP32 accuracy, the mixed form's FP32 phase) or double (FP64 form)
@@ -447,54 +489,81 @@ __device__ __forceinline__ void tile_fJ(const TileCtx<n>& X, const BasisTab& tab
 {
     constexpr bool F64 = sizeof(T) == 8;
     using D = TileDim<n>;
-    using L = TileSm<n, T, F64 ? 5 : 3, 4, 4>;
+    using L = std::conditional_t<F64, Sm64<n>, Sm32<n>>;
     using TB = TileBytes<n, !F64>;
-    constexpr int S = F64 ? 5 : 3, O = S, CS = TileStride<T>::C;
+    constexpr int S = F64 ? 6 : 3, O = S, CS = TileStride<T>::C;
+    static_assert((n - 1) * (n - 1) <= 1 << kDerivExp<n>, "derivatives are scaled into [-1,1]");
     const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
     T* sm = reinterpret_cast<T*>(X.sm);
     uint4* dg = reinterpret_cast<uint4*>(X.sm + L::DIG);
+    if constexpr (F64) {
+        // h_i(r), h_j(s) and their derivatives in fixed point, h_k(t) and h_k'(t) in FP64
+        int2* fx = reinterpret_cast<int2*>(sm);
 #pragma unroll 1
-    for (int d = 0; d < 2; ++d) {
-        T h[n];
-        lagrange_h<n, T>(Tab<T>::xi(tab), Tab<T>::ci(tab), d == 0 ? r[0] : r[1], h);
-        store_dir<n, T>(sm + (d == 0 ? L::HR : L::HS) + lane, d == 1, h);
-    }
-    {
-        T h[n], dh[n];
-        if (jac) {
-            lagrange_hd<n, T>(Tab<T>::xi(tab), Tab<T>::ci(tab), r[2], h, dh);
-            store_dir<n, T>(sm + L::DT + lane, false, dh);
-        } else {
-            lagrange_h<n, T>(Tab<T>::xi(tab), Tab<T>::ci(tab), r[2], h);
+        for (int d = 0; d < 3; ++d) {
+            const T rd = d == 0 ? r[0] : d == 1 ? r[1] : r[2];
+            T h[n], dh[n];
+            if (jac) lagrange_hd<n, T>(tab.xi, tab.ci, rd, h, dh);
+            else lagrange_h<n, T>(tab.xi, tab.ci, rd, h);
+            if (d == 2) {
+                store_dir<n, T>(sm + L::HT + lane, false, h);
+                if (jac) store_dir<n, T>(sm + L::DT + lane, false, dh);
+            } else {
+                int2 v[n];
+#pragma unroll
+                for (int i = 0; i < n; ++i) v[i] = fix60(h[i]);
+                store_dir<n, int2>(fx + (d == 0 ? L::HR : L::HS) + lane, d == 1, v);
+                if (jac) {
+#pragma unroll
+                    for (int i = 0; i < n; ++i) v[i] = fix60(dh[i] * T(pow2<-kDerivExp<n>>()));
+                    store_dir<n, int2>(fx + (d == 0 ? L::DR : L::DS) + lane, d == 1, v);
+                }
+            }
         }
+    } else {
+#pragma unroll 1
+        for (int d = 0; d < 2; ++d) {
+            T h[n];
+            lagrange_h<n, T>(tab.xif, tab.cif, d == 0 ? r[0] : r[1], h);
+            store_dir<n, T>(sm + (d == 0 ? L::HR : L::HS) + lane, d == 1, h);
+        }
+        T h[n], dh[n];
+        lagrange_hd<n, T>(tab.xif, tab.cif, r[2], h, dh);
+        store_dir<n, T>(sm + L::DT + lane, false, dh);
         store_dir<n, T>(sm + L::HT + lane, false, h);
     }
     __syncwarp();
-    constexpr T unit = F64 ? T(1.7763568394002505e-15) : T(1);          // FP64 columns are in units of 2^-49
 #pragma unroll 1
     for (int mt = 0; mt < 2; ++mt) {
         const uint32_t nd = (need >> (16 * mt)) & 0xffffu, hd = tile_heads(X.heads, mt);
         if (!nd) continue;
+        if constexpr (!F64) {
 #pragma unroll 1
-        for (int kc = 0; kc < D::KC; ++kc) {
-            uint32_t a[S][4];
-            tile_left<n, S, T>(sm + L::HR, sm + L::HS, kc, mt, a);
+            for (int kc = 0; kc < D::KC; ++kc) {
+                uint32_t a[S][4];
+                tile_left<n, S, T>(sm + L::HR, sm + L::HS, kc, mt, a);
 #pragma unroll
-            for (int s = 0; s < S; ++s) dg[(kc * S + s) * 32 + lane] = make_uint4(a[s][0], a[s][1], a[s][2], a[s][3]);
+                for (int s = 0; s < S; ++s) dg[(kc * S + s) * 32 + lane] = make_uint4(a[s][0], a[s][1], a[s][2], a[s][3]);
+            }
         }
         // each lane reads back the digits it wrote itself: no barrier
 #pragma unroll 1
         for (int m = 0; m < (jac ? 3 : 1); ++m) {         // x, dx/dr, dx/ds
             float acc[O][D::NT][4];
-            tile_gemm<n, S, O, F64>(
-                [&](int kc, uint32_t (&a)[S][4]) {
+            auto left = [&](int kc, uint32_t (&a)[S][4]) {
+                if constexpr (F64) {
+                    const int2* fx = reinterpret_cast<const int2*>(sm);
+                    tile_left<n, S, int2>(fx + (m == 1 ? L::DR : L::HR), fx + (m == 2 ? L::DS : L::HS), kc, mt, a);
+                } else {
 #pragma unroll
                     for (int s = 0; s < S; ++s) {
                         const uint4 v = dg[(kc * S + s) * 32 + lane];
                         a[s][0] = v.x; a[s][1] = v.y; a[s][2] = v.z; a[s][3] = v.w;
                     }
-                },
-                X.dig + (m == 0 ? 0 : TB::jac + (m - 1) * TB::one), m == 0 ? 5 : TB::SJ, TB::v, hd, nd, X.e, mt, acc);
+                }
+            };
+            tile_gemm<n, S, O>(left, X.dig + (m == 0 || F64 ? 0 : TB::jac + (m - 1) * TB::one), m == 0 || F64 ? TB::SX : 3,
+                               TB::v, hd, nd, X.e, mt, acc);
             T* C = sm + L::C;
 #pragma unroll
             for (int t = 0; t < D::NT; ++t)
@@ -503,27 +572,34 @@ __device__ __forceinline__ void tile_fJ(const TileCtx<n>& X, const BasisTab& tab
                     const int col = 8 * t + 2 * q + (v & 1), row = g + 8 * (v >> 1);
                     if (col < 3 * n) {
                         if constexpr (F64)
-                            C[col * CS + row] = column_f64(acc[0][t][v], acc[1][t][v], acc[2][t][v], acc[3][t][v], acc[4][t][v]);
+                            C[col * CS + row] = column_f64(acc[0][t][v], acc[1][t][v], acc[2][t][v], acc[3][t][v],
+                                                           acc[4][t][v], acc[5][t][v]);
                         else
                             C[col * CS + row] = column(acc[0][t][v], acc[1][t][v], acc[2][t][v]);
                     }
                 }
             __syncwarp();
             T* out = sm + L::OUT + 16 * mt;
-            contract_out<n, T>(out + 3 * m * kTileRows, out + 9 * kTileRows, jac && m == 0, C, sm + L::HT + 16 * mt,
-                               sm + L::DT + 16 * mt, unit);
+            contract_out<n, T>(out + 3 * m * kTileRows, jac && m == 0, C, sm + L::HT + 16 * mt, sm + L::DT + 16 * mt);
             __syncwarp();
         }
     }
-    // from each coordinate's own scale to the element's
+    // from each coordinate's own scale (FP64: and the columns' unit) to the element's
+    constexpr int unit = F64 ? -58 : 0;
     const T* out = sm + L::OUT + lane;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        const T cs = scale_of<T>(X.bx->cscale[a]);
+        const T cs = scale_of<T, unit>(X.bx->cscale[a]);
         x[a] = out[a * kTileRows] * cs;
 #pragma unroll
-        for (int b = 0; b < 3; ++b)
-            J[3 * a + b] = out[(3 + 3 * b + a) * kTileRows] * (b < 2 ? scale_of<T>(X.bx->jscale[b][a]) : cs);
+        for (int b = 0; b < 3; ++b) {
+            T js = cs;
+            if (b < 2) {
+                if constexpr (F64) js = scale_of<T, unit + kDerivExp<n>>(X.bx->cscale[a]);
+                else js = X.bx->jscale[b][a];
+            }
+            J[3 * a + b] = (b < 2 ? out[(3 + 3 * b + a) * kTileRows] : sm[L::DT + a * TileStride<T>::H + lane]) * js;
+        }
     }
     __syncwarp();
 }
@@ -556,7 +632,7 @@ __device__ __forceinline__ void tile_f_df(const TileCtx<n>& X, const BasisTab& t
         const uint32_t nd = (need >> (16 * mt)) & 0xffffu, hd = tile_heads(X.heads, mt);
         if (!nd) continue;
         float acc[5][D::NT][4];
-        tile_gemm<n, 5, 5, false>(
+        tile_gemm<n, 5, 5>(
             [&](int kc, uint32_t (&a)[5][4]) { tile_left<n, 5, float2>(sm + L::HR, sm + L::HS, kc, mt, a); }, X.dig, 5,
             TB::v, hd, nd, X.e, mt, acc);
         float2* C = sm + L::C;
@@ -1364,16 +1440,15 @@ __global__ void __launch_bounds__(TileLB<KIND>::threads, TileLB<KIND>::blocks) k
 }
 
 // ---- set-up: the digits, scales and affine deviation of every element ----
-// One block per element.  Shared memory: the scaled node offsets in FP64 and
-// (mixed form) FP32, and one direction's derivative values; planes of constant
+// One block per element.  Shared memory: the scaled node offsets in FP64 and,
+// mixed form, in FP32 and one direction's derivative values; planes of constant
 // k are PL apart so that the fragments' reads of one column per k fall into
 // distinct banks.  The derivative of the nodal values is taken in the
 // precision its digits hold.
 template <int n, bool MIXED>
 struct DigitsSm {
-    using TJ = std::conditional_t<MIXED, float, double>;
     static constexpr int PL = n * n + (40 - n * n % 32) % 32, V = 3 * n * PL;
-    static constexpr int bytes = V * (int)(sizeof(double) + (MIXED ? 2 : 1) * sizeof(TJ)) + n * n * (int)sizeof(TJ);
+    static constexpr int bytes = V * (int)(sizeof(double) + (MIXED ? 2 * sizeof(float) : 0)) + (MIXED ? n * n * (int)sizeof(float) : 0);
 };
 
 // exponent of a magnitude, so that v < 2^(exponent - 1022); integer maxima of
@@ -1391,24 +1466,18 @@ __global__ void __launch_bounds__(128) k_digits(int64_t E, const double* __restr
     using D = TileDim<n>;
     using TB = TileBytes<n, MIXED>;
     using L = DigitsSm<n, MIXED>;
-    using TJ = typename L::TJ;
     constexpr int n3 = n * n * n, PL = L::PL;
     extern __shared__ double digits_sm[];
     double* V = digits_sm;
-    TJ* W = reinterpret_cast<TJ*>(V + L::V);
-    TJ* Vj = MIXED ? W + L::V : reinterpret_cast<TJ*>(V);
-    TJ* der = W + (MIXED ? 2 : 1) * L::V;                 // der[i n + m] = h_m'(xi_i)
+    float* W = reinterpret_cast<float*>(V + L::V);        // (mixed form)
+    float* Vj = W + L::V;
+    float* der = Vj + L::V;                               // der[i n + m] = h_m'(xi_i)
     __shared__ int4 red[4];
     const int64_t e = blockIdx.x;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (threadIdx.x < n) {
-        TJ h[n], d[n], xi[n], ci[n];
-#pragma unroll
-        for (int m = 0; m < n; ++m) {
-            xi[m] = (TJ)tab.xi[m];
-            ci[m] = (TJ)tab.ci[m];
-        }
-        lagrange_hd<n, TJ>(xi, ci, (TJ)tab.xi[threadIdx.x], h, d);
+    if (MIXED && threadIdx.x < n) {
+        float h[n], d[n];
+        lagrange_hd<n, float>(tab.xif, tab.cif, tab.xif[threadIdx.x], h, d);
 #pragma unroll
         for (int m = 0; m < n; ++m) der[threadIdx.x * n + m] = d[m];
     }
@@ -1460,51 +1529,50 @@ __global__ void __launch_bounds__(128) k_digits(int64_t E, const double* __restr
         const int a = i / (n * PL);
         const double v = V[i] * ldexp(1.0, -(a == 0 ? ea.x : a == 1 ? ea.y : ea.z));
         V[i] = v;
-        if (MIXED) Vj[i] = (TJ)v;
+        if (MIXED) Vj[i] = (float)v;
     }
     __syncthreads();
-    // digits of the values val[], each coordinate divided by its power of two
+    // digits of the values val[], each coordinate divided by its power of two;
+    // FP64 values give 6, of which SD are kept
     auto frags = [&](auto* val, int3 sa, unsigned char* out, auto digits) {
         constexpr int SD = decltype(digits)::value;
-        using TV = std::conditional_t<SD == 5, double, float>;
+        using TV = std::remove_pointer_t<decltype(val)>;
         for (int f = warp; f < D::KC * D::NT; f += 4) {
             const int kc = f / D::NT, t = f % D::NT, g = lane >> 2, q = lane & 3;
             const int col = 8 * t + g;                    // column a n + k is plane a n + k
-            const TV ji = ldexp(TV(1), -(col < n ? sa.x : col < 2 * n ? sa.y : sa.z));
-            uint32_t b[5][2];
+            RightFrag<SD> R;
 #pragma unroll
             for (int hf = 0; hf < 2; ++hf) {
                 TV v[2];
 #pragma unroll
                 for (int u = 0; u < 2; ++u) {
                     const int kap = 16 * kc + 8 * hf + 2 * q + u;
-                    v[u] = kap < D::n2 && col < 3 * n ? (TV)val[col * PL + kap] : TV(0);
+                    v[u] = kap < D::n2 && col < 3 * n ? val[col * PL + kap] : TV(0);
                 }
-                uint32_t d[SD];
-                digits2(v[0], ji, v[1], ji, d);
+                uint32_t d[sizeof(TV) == 8 ? 6 : 3];
+                if constexpr (sizeof(TV) == 8) {
+                    const int2 one = make_int2(1 << 30, 0);   // (|v| < 1/2, scaled already)
+                    digits2(fix60(v[0]), one, fix60(v[1]), one, d);
+                } else {
+                    const float ji = ldexpf(1.0f, -(col < n ? sa.x : col < 2 * n ? sa.y : sa.z));
+                    digits2(v[0], ji, v[1], ji, d);
+                }
 #pragma unroll
-                for (int s = 0; s < SD; ++s) b[s][hf] = d[s];
+                for (int s = 0; s < SD; ++s) R.b[s][hf] = d[s];
             }
-            unsigned char* F = out + (int64_t)f * FragBytes<SD>::v;
-            reinterpret_cast<uint4*>(F)[lane] = make_uint4(b[0][0], b[0][1], b[1][0], b[1][1]);
-            if constexpr (SD == 5) {
-                reinterpret_cast<uint4*>(F + 512)[lane] = make_uint4(b[2][0], b[2][1], b[3][0], b[3][1]);
-                reinterpret_cast<uint2*>(F + 1024)[lane] = make_uint2(b[4][0], b[4][1]);
-            } else {
-                reinterpret_cast<uint2*>(F + 512)[lane] = make_uint2(b[2][0], b[2][1]);
-            }
+            R.store(out + (int64_t)f * FragBytes<SD>::v);
         }
     };
     unsigned char* out = dig + e * TB::v;
-    frags(V, make_int3(0, 0, 0), out, std::integral_constant<int, 5>());
-    // dx/dr and dx/ds, each coordinate with its own power of two
+    frags(V, make_int3(0, 0, 0), out, std::integral_constant<int, TB::SX>());
+    // mixed form: dx/dr and dx/ds, each coordinate with its own power of two
 #pragma unroll 1
-    for (int m = 0; m < 2; ++m) {
+    for (int m = 0; MIXED && m < 2; ++m) {
         most = make_int4(0, 0, 0, 0);
         for (int i = threadIdx.x; i < 3 * n3; i += 128) {
             const int c = i / (n * n), q = i % (n * n), at = m == 0 ? q % n : q / n, st = m == 0 ? 1 : n;
-            const TJ* v = Vj + c * PL + q - at * st;
-            TJ w = TJ(0);
+            const float* v = Vj + c * PL + q - at * st;
+            float w = 0.0f;
 #pragma unroll
             for (int u = 0; u < n; ++u) w += der[at * n + u] * v[u * st];
             W[c * PL + q] = w;
@@ -1515,7 +1583,7 @@ __global__ void __launch_bounds__(128) k_digits(int64_t E, const double* __restr
         }
         most = block_max(most);
         const int3 sa = make_int3(scale_exp(most.x, -100), scale_exp(most.y, -100), scale_exp(most.z, -100));
-        frags(W, sa, out + TB::jac + m * TB::one, std::integral_constant<int, TB::SJ>());
+        frags(W, sa, out + TB::jac + m * TB::one, std::integral_constant<int, 3>());
         if (threadIdx.x == 0) {
             boxes[e].jscale[m][0] = ldexpf(1.0f, sa.x + ea.x - ex);
             boxes[e].jscale[m][1] = ldexpf(1.0f, sa.y + ea.y - ex);
