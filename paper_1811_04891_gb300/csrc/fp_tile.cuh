@@ -27,8 +27,10 @@
 // against extended precision, relative to half the element's width, N = 7,
 // width 0.1: 2e-16 rms; by FP64 sum factorisation 3e-16 for coordinates
 // around zero, 3e-15 around 0.5; with 5 digits 3e-15).  Mixed form: 5 digits
-// and orders 0..4, about 2^-48 (compensated residuals), 3 digits and orders
-// 0..2, about 2^-27 (its FP32 phase).  A row's sums do not depend on the other
+// and orders 0..5 for its compensated residuals (1.6e-14 rms, of which 1.5e-14
+// from the double-float basis; 1.7e-14 on float pairs of the coordinates,
+// 2.0e-14 without order 5), 3 digits and orders 0..2, about 2^-27, for its
+// FP32 phase.  A row's sums do not depend on the other
 // rows, so a pair's result does not depend on which pairs share its warp, on
 // the block size, or on the entry point.
 //
@@ -272,8 +274,9 @@ struct RightFrag {
 };
 
 // acc[o][t] += the order-o products of S left digits and the S right digits of
-// tile t
-template <int n, int S, int O>
+// tile t; FINE: order S joins the sums of order S - 1, its right digits scaled
+// by 2^-10
+template <int n, int S, int O, bool FINE>
 __device__ __forceinline__ void mma_digits(const uint32_t (&a)[S][4], const RightFrag<S>& R, int t,
                                            float (&acc)[O][TileDim<n>::NT][4])
 {
@@ -282,6 +285,13 @@ __device__ __forceinline__ void mma_digits(const uint32_t (&a)[S][4], const Righ
 #pragma unroll
         for (int s = 0; s < S; ++s)
             if (s + u < O) mma_16816(acc[s + u][t], a[s], R.b[u][0], R.b[u][1]);
+    if constexpr (FINE) {
+        static_assert(O == S, "the next order is S");
+        const __half2 sc = __floats2half2_rn(pow2<-10>(), pow2<-10>());
+        auto down = [&](uint32_t d) { return h2bits(__hmul2(*reinterpret_cast<const __half2*>(&d), sc)); };
+#pragma unroll
+        for (int u = 1; u < S; ++u) mma_16816(acc[S - 1][t], a[S - u], down(R.b[u][0]), down(R.b[u][1]));
+    }
 }
 
 // acc = the digit products of a 16-row tile over all k16 steps.  left(kc, a)
@@ -290,7 +300,7 @@ __device__ __forceinline__ void mma_digits(const uint32_t (&a)[S][4], const Righ
 // fetched while the current ones are multiplied (three digits: they fit the
 // registers).  Several: each element's rows in turn, the others masked to
 // zero.
-template <int n, int S, int O, typename Left>
+template <int n, int S, int O, bool FINE, typename Left>
 __device__ __forceinline__ void tile_gemm(Left&& left, const unsigned char* __restrict__ base, int sb, int64_t ebytes,
                                           uint32_t heads, uint32_t need, int e, int mt,
                                           float (&acc)[O][TileDim<n>::NT][4])
@@ -331,7 +341,7 @@ __device__ __forceinline__ void tile_gemm(Left&& left, const unsigned char* __re
                 uint32_t a[S][4];
                 left(kc, a);
 #pragma unroll
-                for (int t = 0; t < D::NT; ++t) mma_digits<n, S, O>(a, R[t], t, acc);
+                for (int t = 0; t < D::NT; ++t) mma_digits<n, S, O, FINE>(a, R[t], t, acc);
             }
             return;
         }
@@ -362,14 +372,14 @@ __device__ __forceinline__ void tile_gemm(Left&& left, const unsigned char* __re
                 for (int t = 0; t < D::NT; ++t) R[t] = next[t];
                 if (hm || kc + 1 < D::KC) fetch(frag(__ffs(hm ? hm : hs) - 1, hm ? kc : kc + 1));
 #pragma unroll
-                for (int t = 0; t < D::NT; ++t) mma_digits<n, S, O>(am, R[t], t, acc);
+                for (int t = 0; t < D::NT; ++t) mma_digits<n, S, O, FINE>(am, R[t], t, acc);
             } else {
                 const unsigned char* F = frag(h, kc);
 #pragma unroll
                 for (int t = 0; t < D::NT; ++t) {
                     RightFrag<S> R;
                     R.load(F + t * FragBytes<1>::v * sb, sb);
-                    mma_digits<n, S, O>(am, R, t, acc);
+                    mma_digits<n, S, O, FINE>(am, R, t, acc);
                 }
             }
         }
@@ -562,7 +572,7 @@ __device__ __forceinline__ void tile_fJ(const TileCtx<n>& X, const BasisTab& tab
                     }
                 }
             };
-            tile_gemm<n, S, O>(left, X.dig + (m == 0 || F64 ? 0 : TB::jac + (m - 1) * TB::one), m == 0 || F64 ? TB::SX : 3,
+            tile_gemm<n, S, O, false>(left, X.dig + (m == 0 || F64 ? 0 : TB::jac + (m - 1) * TB::one), m == 0 || F64 ? TB::SX : 3,
                                TB::v, hd, nd, X.e, mt, acc);
             T* C = sm + L::C;
 #pragma unroll
@@ -632,7 +642,7 @@ __device__ __forceinline__ void tile_f_df(const TileCtx<n>& X, const BasisTab& t
         const uint32_t nd = (need >> (16 * mt)) & 0xffffu, hd = tile_heads(X.heads, mt);
         if (!nd) continue;
         float acc[5][D::NT][4];
-        tile_gemm<n, 5, 5>(
+        tile_gemm<n, 5, 5, true>(
             [&](int kc, uint32_t (&a)[5][4]) { tile_left<n, 5, float2>(sm + L::HR, sm + L::HS, kc, mt, a); }, X.dig, 5,
             TB::v, hd, nd, X.e, mt, acc);
         float2* C = sm + L::C;
