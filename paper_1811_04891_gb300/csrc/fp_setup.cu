@@ -11,6 +11,7 @@
 //              from box overlap (count, scan, fill, per-cell sort).
 //  k_face_* / k_dist_default  default nodal distance-to-boundary field D^k.
 #include <algorithm>
+#include <climits>
 
 #include "fp_common.cuh"
 #include "fp_internal.h"
@@ -21,23 +22,38 @@ namespace fpg {
 // k_hull: one block per element.  Dynamic shared memory: 4 * n^3 doubles
 // (three Bernstein coefficient arrays + one transform buffer).
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ double block_reduce_min(double v, double* sh)
+// Minima and maxima go by the order of the bits as signed integers: an FP64
+// minimum takes the FP64 pipe, which bounds this kernel, 16 clocks of an SM a
+// warp.  (32,768 elements of order 7: 4.77 ms with FP64 minima, a third of the
+// kernel's operations.)  The coordinates are finite.
+__device__ __forceinline__ long long order_key(double v)
+{
+    const long long b = __double_as_longlong(v);
+    return b ^ ((b >> 63) & 0x7fffffffffffffffLL);
+}
+
+__device__ __forceinline__ double key_value(long long k)
+{
+    return __longlong_as_double(k ^ ((k >> 63) & 0x7fffffffffffffffLL));
+}
+
+__device__ __forceinline__ long long block_reduce_max(long long v, long long* sh)
 {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fmin(v, __shfl_xor_sync(0xffffffffu, v, o));
+    for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
     const int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = (blockDim.x + 31) >> 5;
     __syncthreads();
     if (l == 0) sh[w] = v;
     __syncthreads();
-    double r = sh[0];
-    for (int i = 1; i < nw; ++i) r = fmin(r, sh[i]);
+    long long r = sh[0];
+    for (int i = 1; i < nw; ++i) r = max(r, sh[i]);
     __syncthreads();
     return r;
 }
 
-__device__ __forceinline__ double block_reduce_max(double v, double* sh)
+__device__ __forceinline__ long long block_reduce_min(long long v, long long* sh)
 {
-    return -block_reduce_min(-v, sh);
+    return ~block_reduce_max(~v, sh);
 }
 
 __global__ void k_hull(int n, int64_t E, const double* __restrict__ coords,
@@ -45,7 +61,7 @@ __global__ void k_hull(int n, int64_t E, const double* __restrict__ coords,
                        ElemBox* __restrict__ boxes, double* __restrict__ nodebox)
 {
     extern __shared__ double sm[];
-    __shared__ double red[32];
+    __shared__ long long red[32];
     __shared__ double frame[12];
     const int n3 = n * n * n;
     const int64_t e = blockIdx.x;
@@ -54,17 +70,18 @@ __global__ void k_hull(int n, int64_t E, const double* __restrict__ coords,
     const int N = n - 1;
 
     // node box and h_e (no FMA contraction: matches a plain evaluation)
-    double lo[3], hi[3], cmax = 0.0;
+    double lo[3], hi[3];
+    long long cmost = 0;
     for (int a = 0; a < 3; ++a) {
         const double* X = coords + ((int64_t)a * E + e) * n3;
-        double mn = INFINITY, mx = -INFINITY;
+        long long mn = LLONG_MAX, mx = LLONG_MIN;
         for (int q = threadIdx.x; q < n3; q += blockDim.x) {
-            double v = X[q];
-            mn = fmin(mn, v);
-            mx = fmax(mx, v);
+            const long long v = order_key(X[q]);
+            mn = min(mn, v);
+            mx = max(mx, v);
         }
-        lo[a] = block_reduce_min(mn, red);
-        hi[a] = block_reduce_max(mx, red);
+        lo[a] = key_value(block_reduce_min(mn, red));
+        hi[a] = key_value(block_reduce_max(mx, red));
     }
     const double dx = hi[0] - lo[0], dy = hi[1] - lo[1], dz = hi[2] - lo[2];
     const double he = sqrt(__dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz)));
@@ -128,13 +145,11 @@ __global__ void k_hull(int n, int64_t E, const double* __restrict__ coords,
     // i, then j, then k (tensor-product change of basis)
     for (int a = 0; a < 3; ++a) {
         const double* X = coords + ((int64_t)a * E + e) * n3;
-        double m = 0.0;
         for (int q = threadIdx.x; q < n3; q += blockDim.x) {
             double v = X[q] - c[a];
             tmp[q] = v;
-            m = fmax(m, fabs(v));
+            cmost = max(cmost, order_key(fabs(v)));
         }
-        cmax = fmax(cmax, m);
         __syncthreads();
         for (int q = threadIdx.x; q < n3; q += blockDim.x) {        // along i
             int i = q % n, rest = q / n;
@@ -158,29 +173,34 @@ __global__ void k_hull(int n, int64_t E, const double* __restrict__ coords,
         }
         __syncthreads();
     }
-    cmax = block_reduce_max(cmax, red);
+    const double cmax = key_value(block_reduce_max(cmost, red));
 
     // boxes of the control points: axis box of c + B, frame box of Ai B
     double Ai[9];
     for (int q = 0; q < 9; ++q) Ai[q] = frame[3 + q];
-    double amin[3] = {INFINITY, INFINITY, INFINITY}, amax[3] = {-INFINITY, -INFINITY, -INFINITY};
-    double omin[3] = {INFINITY, INFINITY, INFINITY}, omax[3] = {-INFINITY, -INFINITY, -INFINITY};
+    long long least[6], most[6];                          // axis box, frame box
+    for (int a = 0; a < 6; ++a) {
+        least[a] = LLONG_MAX;
+        most[a] = LLONG_MIN;
+    }
     for (int q = threadIdx.x; q < n3; q += blockDim.x) {
         double b0 = B[0][q], b1 = B[1][q], b2 = B[2][q];
         double bb[3] = {b0, b1, b2};
         for (int a = 0; a < 3; ++a) {
-            amin[a] = fmin(amin[a], bb[a]);
-            amax[a] = fmax(amax[a], bb[a]);
             double y = Ai[3 * a] * b0 + Ai[3 * a + 1] * b1 + Ai[3 * a + 2] * b2;
-            omin[a] = fmin(omin[a], y);
-            omax[a] = fmax(omax[a], y);
+            const long long kb = order_key(bb[a]), ky = order_key(y);
+            least[a] = min(least[a], kb);
+            most[a] = max(most[a], kb);
+            least[3 + a] = min(least[3 + a], ky);
+            most[3 + a] = max(most[3 + a], ky);
         }
     }
+    double amin[3], amax[3], omin[3], omax[3];
     for (int a = 0; a < 3; ++a) {
-        amin[a] = block_reduce_min(amin[a], red);
-        amax[a] = block_reduce_max(amax[a], red);
-        omin[a] = block_reduce_min(omin[a], red);
-        omax[a] = block_reduce_max(omax[a], red);
+        amin[a] = key_value(block_reduce_min(least[a], red));
+        amax[a] = key_value(block_reduce_max(most[a], red));
+        omin[a] = key_value(block_reduce_min(least[3 + a], red));
+        omax[a] = key_value(block_reduce_max(most[3 + a], red));
     }
     if (threadIdx.x == 0) {
         ElemBox bx;
@@ -216,7 +236,7 @@ __global__ void k_hull(int n, int64_t E, const double* __restrict__ coords,
 __global__ void k_reduce_boxes(int64_t E, const ElemBox* __restrict__ boxes,
                                const double* __restrict__ nodebox, double* __restrict__ out)
 {
-    __shared__ double red[32];
+    __shared__ long long red[32];
     double v[12];
     for (int a = 0; a < 3; ++a) {
         v[a] = INFINITY; v[3 + a] = -INFINITY; v[6 + a] = INFINITY; v[9 + a] = -INFINITY;
@@ -231,8 +251,8 @@ __global__ void k_reduce_boxes(int64_t E, const ElemBox* __restrict__ boxes,
     }
     for (int q = 0; q < 12; ++q) {
         bool ismin = (q % 6) < 3;
-        double r = ismin ? block_reduce_min(v[q], red) : block_reduce_max(v[q], red);
-        if (threadIdx.x == 0) out[12 * blockIdx.x + q] = r;
+        const long long k = order_key(v[q]), r = ismin ? block_reduce_min(k, red) : block_reduce_max(k, red);
+        if (threadIdx.x == 0) out[12 * blockIdx.x + q] = key_value(r);
     }
 }
 
