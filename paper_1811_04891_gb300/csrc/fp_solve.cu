@@ -120,8 +120,18 @@ __global__ void __launch_bounds__(128) k_newton_resume(NewtonArgs A, BasisTab ta
 }
 
 // passes 1 and 2 in one kernel: the FP32 work of some warps overlaps the
-// FP64 work of others (the orders without a tile kernel; the compiler is left
-// free in its registers).
+// FP64 work of others (the orders without a tile kernel).
+// Its launch shape.  CAP (blocks of up to 128 threads, n <= 10, where 128
+// registers need no spills): registers capped so that four blocks of 128
+// threads fit an SM.  Otherwise (persistent grids of the workspace calls,
+// larger n) the compiler takes what it wants, 222 registers at n = 13; that
+// has to be asked for by the block count: left out, 128 are used and a find
+// of 10,000 points in 512 elements of order 12 takes 960 us instead of 838.
+template <int n, bool CAP> struct MixedLB {
+    static constexpr int threads = CAP ? 128 : 256;
+    static constexpr int blocks = CAP ? 4 : 1;
+};
+
 template <int n>
 __device__ __forceinline__ void solve_mixed(const NewtonArgs& A, const BasisTab& tab, int64_t s, int32_t* fbl,
                                             int64_t fbc)
@@ -236,8 +246,8 @@ __device__ __forceinline__ void solve_mixed(const NewtonArgs& A, const BasisTab&
     }
 }
 
-template <int n>
-__global__ void __launch_bounds__(256)
+template <int n, bool CAP>
+__global__ void __launch_bounds__(MixedLB<n, CAP>::threads, MixedLB<n, CAP>::blocks)
     k_newton_mixed(NewtonArgs A, BasisTab tab)
 {
     const PairRange R = pair_range(A);
@@ -418,7 +428,14 @@ static cudaError_t newton_form(const FindArgs& a, int64_t npairs, const BasisTab
     } else {
         if (grid == 0) grid = grid_for(npairs, block, a.persistent_blocks);
         if constexpr (MIXED) {
-            k_newton_mixed<n><<<grid, block, 0, s>>>(na, tab);
+            bool capped = false;
+            if constexpr (n <= 10) {
+                if (block <= 128 && (a.persistent_blocks == 0 || a.queue)) {
+                    k_newton_mixed<n, true><<<grid, block, 0, s>>>(na, tab);
+                    capped = true;
+                }
+            }
+            if (!capped) k_newton_mixed<n, false><<<grid, block, 0, s>>>(na, tab);
         } else {
             na.pstate = a.pstate;
             k_newton<n><<<grid, block, 0, s>>>(na, tab);
@@ -507,7 +524,9 @@ static int newton_fit_form(int block)
     } else {
         int k = 0;
         cudaError_t e;
-        if constexpr (MIXED) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&k, k_newton_mixed<n>, block, 0);
+        if constexpr (MIXED)
+            e = block <= 128 && n <= 10 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&k, k_newton_mixed<n, n <= 10>, block, 0)
+                                        : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&k, k_newton_mixed<n, false>, block, 0);
         else e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&k, k_newton<n>, block, 0);
         return e == cudaSuccess ? k : 1;
     }
