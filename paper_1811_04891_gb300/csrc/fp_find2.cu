@@ -683,7 +683,7 @@ struct Newton2Args {
     int max_newton;
     const int32_t* warm_elem;
     const double* warm_rst;
-    int32_t* list;             // [P] sorted positions left to k_newton2_listed
+    int32_t* list;             // [P] sorted positions left to k_newton2_listed; null: no FP32 starts, no list
     int32_t* count;
 };
 
@@ -699,7 +699,15 @@ struct Newton2Args {
 // the same warps they would keep the other lanes waiting.
 // 1.5e6 points in 16,384 elements of order 7, whole find and evaluation:
 // 10,300 us with every solve from the nearest node, 7,100 us.
+// Few pairs, or few of an element, have every solve start at the nearest node,
+// in one launch: the time is then one solve's chain, to which the FP32 steps
+// and the second launch add.  N = 7, nearest node / FP32 start in us:
+//   64 elements       10,000 points 432/463     50,000 741/606    200,000 1861/1036
+//   1,024 elements    10,000 points 364/406     50,000 545/512    200,000 1169/854
+//   16,384 elements   10,000 points 305/390     50,000 517/694    200,000 1401/1367
+// (The two starts lead to the same root; r agrees to the solves' tolerance.)
 constexpr double kAffineSeed2 = 0.25;
+constexpr int64_t kStart32Pairs = 40000, kStart32PerElem = 10;
 
 template <int n>
 __device__ __forceinline__ bool start32(const ElemBox& bx, const float* __restrict__ V0, const float* __restrict__ V1,
@@ -778,13 +786,14 @@ __device__ __forceinline__ void solve_pair2(const Newton2Args& A, const BasisTab
                 ready = true;
             }
         }
-        if (!ready)
+        if (!ready && A.list) {
             ready = start32<n>(A.boxes[e], A.coords32 + (int64_t)e * n2, A.coords32 + (A.E + e) * n2, tab, xs, r);
-        if (!ready) {
-            const int k = atomicAdd(A.count, 1);
-            if (k < A.P) {                   // the list's room; past it the solve is done here
-                A.list[k] = (int32_t)s;
-                return;
+            if (!ready) {
+                const int k = atomicAdd(A.count, 1);
+                if (k < A.P) {               // the list's room; past it the solve is done here
+                    A.list[k] = (int32_t)s;
+                    return;
+                }
             }
         }
     }
@@ -938,14 +947,17 @@ static cudaError_t solve2_n(const FindArgs& a, int64_t npairs, const BasisTab& t
         if (a.ev[2]) cudaEventRecord(a.ev[2], s);
         // the per-point counts (free after the scan) hold the list, a scan
         // scratch word (free after the sort) its length
-        na.list = a.cnt;
+        const bool listed = npairs > kStart32Pairs && npairs >= kStart32PerElem * a.E;
+        na.list = listed ? a.cnt : nullptr;
         na.count = a.scan_tmp;
-        cudaError_t err = cudaMemsetAsync(na.count, 0, sizeof(int32_t), s);
+        cudaError_t err = listed ? cudaMemsetAsync(na.count, 0, sizeof(int32_t), s) : cudaSuccess;
         if (err != cudaSuccess) return err;
         k_newton2<n><<<grid, block, 0, s>>>(na, tab);
-        k_newton2_listed<n><<<std::max(1u, std::min(grid, 8192u)), block, 0, s>>>(na, tab);
         count_launch();
-        count_launch();
+        if (listed) {
+            k_newton2_listed<n><<<std::max(1u, std::min(grid, 8192u)), block, 0, s>>>(na, tab);
+            count_launch();
+        }
         err = cudaGetLastError();
         if (err != cudaSuccess) return err;
         if (a.ev[3]) cudaEventRecord(a.ev[3], s);
