@@ -653,14 +653,16 @@ cudaError_t launch_eval_pairs(int n, int64_t E, int64_t P, const int32_t* dcount
     const bool df = ev.fdf != nullptr;
     const int64_t stage_bytes = (int64_t)ev.F * n * n * n * (int64_t)sizeof(float2);
     const bool staged = df && ev.staged && stage_bytes <= kStageMaxBytes;
-    const bool planes = !s_lo && P <= kPlanePairs, split = !s_lo && P <= kSplitPairs && n >= kSplitMinN && ev.F <= kSplitFields;
+    // (the staging that a caller asked for comes first)
+    const bool planes = !s_lo && !staged && P <= kPlanePairs;
+    const bool split = !s_lo && !staged && P <= kSplitPairs && n >= kSplitMinN && ev.F <= kSplitFields;
     const dim3 grid2(grid, split ? ev.F : 1);
     switch (n) {
 #define FP_CASE(NN)                                                                       \
     case NN:                                                                              \
         if (planes && df) k_eval_pairs_planes<NN, PlanesDf><<<grid * kPlaneGroup<NN>, 128, 0, s>>>(a, ev.fdf, tab); \
         else if (planes) k_eval_pairs_planes<NN, PlanesF64><<<grid * kPlaneGroup<NN>, 128, 0, s>>>(a, ev.f64, tab); \
-        else if (staged && !split) k_eval_pairs_staged<NN><<<grid, kStageTile, stage_bytes, s>>>(a, tab); \
+        else if (staged) k_eval_pairs_staged<NN><<<grid, kStageTile, stage_bytes, s>>>(a, tab); \
         else if (df) k_eval_pairs<NN, true><<<grid2, 128, 0, s>>>(a, tab);                \
         else k_eval_pairs<NN, false><<<grid2, 128, 0, s>>>(a, tab);                       \
         break;
