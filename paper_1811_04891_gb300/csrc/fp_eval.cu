@@ -248,21 +248,53 @@ __global__ void __launch_bounds__(128) k_eval(EvalArgs A, BasisTab tab)
 // calls with at most this many (point, field) values take one thread each
 constexpr int64_t kSplitEval = int64_t(1) << 21;
 
-// Calls with at most this many (point, field) values (fused: points) evaluate
-// by planes.  us, one thread per value / planes, N = 7: 2,000 values 38/16,
-// 10,000 values 40/22, 40,000 values 73/52 at random points; but where
-// neighbouring points share their element, 131,072 values take 49/141.
-// Sorted pairs, whole find and evaluation of 4 posted fields: 2,000 points
-// 259/188, 10,000 361/270, 40,000 418/435.
-constexpr int64_t kPlaneValues = 20000, kPlanePairs = 20000;
+// Which calls evaluate by planes.  A group takes its point's fields one after
+// the other, and the groups of n >= 9 leave up to 7 of 16 lanes idle, so it is
+// for few values of few fields (more of them where the chain of one thread is
+// long).  us, one thread per value / planes, points of one element side by
+// side (points in any order gain more, up to twice as much):
+//   FP64    n = 3    F = 3: 2,000 points 6/5;  F = 6: 2,000 6/7
+//           n = 8    F = 1: 2,000 points 34/7, 10,000 34/21, 20,000 47/37;  F = 6: 2,000 36/25;  F = 12: 500 37/46
+//           n = 10   F = 1: 5,000 54/29, 10,000 55/51;  F = 3: 5,000 57/64;  F = 6: 2,000 58/49;  F = 12: 500 59/64
+//           n = 13   F = 6: 2,000 121/78;  F = 12: 500 158/113
+//   posted  n = 8    F = 1: 2,000 24/8, 20,000 32/29;  F = 3: 5,000 27/27;  F = 12: 500 32/42
+//           n = 10   F = 3: 5,000 44/37;  F = 6: 2,000 47/35;  F = 12: 500 65/54
+static bool eval_by_planes(int n, int64_t P, int F, bool df)
+{
+    const int fields = n <= 3 ? 4 : n <= 9 || (n == 10 && !df) ? 6 : 12;
+    return F <= fields && P * F <= (n <= 8 ? 20000 : df ? 15000 : 12000);
+}
 
-// Calls with at most this many points take one thread per sorted pair and
-// field, at n = 6 and above: find and evaluation of 4 posted fields at N = 7,
-// 40,000 points 424 -> 383 us (N = 9 684 -> 640, FP64 fields 933 -> 902); with
-// 130,000 the basis of every field costs more than the threads give (642 ->
-// 679), at N = 3 already with 40,000 (196 -> 208).
-constexpr int64_t kSplitPairs = 65536;
-constexpr int kSplitFields = 16, kSplitMinN = 6;
+// Posted points in thread form share their rows' loads (see
+// k_eval_points_df).  us, thread / planes, points of one element side by side:
+//   n = 6    F = 1: 2,000 points 10/4, 20,000 11/8;  F = 3: 5,000 11/7;  F = 6: 500 10/10
+//   n = 8    F = 1: 2,000 17/5, 10,000 18/13, 20,000 18/22;  F = 3: 2,000 17/12, 5,000 18/21;  F = 6: 500 17/21
+//   n = 10   F = 1: 2,000 36/7, 20,000 38/33;  F = 3: 5,000 37/27;  F = 6: 2,000 37/29
+//   n = 13   F = 1: 2,000 69/15, 20,000 75/69;  F = 6: 2,000 72/79 (in any order 141/92)
+static bool points_by_planes(int n, int64_t P, int F)
+{
+    return F <= (n <= 9 ? 3 : 6) && P * F <= (n == 8 ? 10000 : 20000);
+}
+
+// Sorted pairs of a find (thread / planes / one thread per pair and field, us):
+//   FP64    n = 6    F = 3: 20,000 points 60/49/48, 65,000 114/147/127
+//           n = 8    F = 3: 20,000 126/79/94, 40,000 185/148/172, 65,000 246/241/258
+//           n = 10   F = 1: 5,000 59/30/59, 20,000 84/101/84;  F = 6: 2,000 332/49/64, 5,000 321/117/86, 65,000 868/1287/857
+//   posted  n = 6    F = 3: 20,000 38/24/34, 40,000 46/39/50, 65,000 55/59/71
+//           n = 7    F = 3: 40,000 82/58/71, 65,000 93/81/94;  F = 6: 65,000 161/149/157
+//           n = 8    F = 3: 10,000 104/42/52, 20,000 102/72/65, 40,000 115/122/90, 65,000 123/193/114;  F = 12: 5,000 512/86/78
+//           n = 13   F = 6: 2,000 408/146/99, 20,000 385/500/226, 65,000 631/1335/550
+// The basis of every field costs more than the threads give once the pairs
+// fill the GPU several times, sooner the lower the order.
+enum PairForm { PAIR_THREAD, PAIR_PLANES, PAIR_FIELD };
+constexpr int kFieldMinN = 7;
+
+static PairForm pair_form(int n, int64_t P, int F, bool df)
+{
+    if (n >= 9 ? P * F <= (df ? 10000 : n >= 12 ? 15000 : 12000) : P <= 20000 && !(df && n == 8 && P * F > 30000))
+        return PAIR_PLANES;
+    return n >= kFieldMinN && F <= 16 && P <= (df || n >= 9 ? 65536 : 50000) ? PAIR_FIELD : PAIR_THREAD;
+}
 
 template <int n>
 static unsigned plane_grid(int64_t count)
@@ -275,7 +307,7 @@ cudaError_t launch_eval(int n, int64_t E, int64_t P, const int32_t* code, const 
 {
     if (P == 0) return cudaSuccess;
     EvalArgs a{E, P, code, elem, rst, F, fields, out};
-    const bool split = P * F <= kSplitEval, planes = P * F <= kPlaneValues;
+    const bool split = P * F <= kSplitEval, planes = eval_by_planes(n, P, F, false);
     const unsigned grid = (unsigned)(((split ? P * F : P) + 127) / 128);
     switch (n) {
 #define FP_CASE(NN)                                                                                           \
@@ -453,7 +485,7 @@ cudaError_t launch_eval_points_df(int n, int64_t E, int64_t P, int F, const int3
 {
     if (P == 0) return cudaSuccess;
     const unsigned grid = value_blocks(P) * F;
-    const bool planes = P * F <= kPlaneValues;
+    const bool planes = points_by_planes(n, P, F);
     switch (n) {
 #define FP_CASE(NN)                                                                                           \
     case NN:                                                                                                  \
@@ -474,7 +506,7 @@ cudaError_t launch_eval_df(int n, int64_t E, int64_t P, const int32_t* code, con
 {
     if (P == 0) return cudaSuccess;
     Eval2Args a{E, P, code, elem, rst, F, fields, out};
-    const bool split = P * F <= kSplitEval, planes = P * F <= kPlaneValues;
+    const bool split = P * F <= kSplitEval, planes = eval_by_planes(n, P, F, true);
     const unsigned grid = (unsigned)(((split ? P * F : P) + 127) / 128);
     switch (n) {
 #define FP_CASE(NN)                                                     \
@@ -536,12 +568,14 @@ __device__ __forceinline__ void eval_point_df(const float2* __restrict__ Fdf, in
 }
 
 
-// one thread per winning pair, or (gridDim.y = F) one per pair and field
-template <int n, bool DF>
+// one thread per winning pair, or (FIELD, gridDim.y = F) one per pair and
+// field; a kernel of its own each, which leaves the compiler its registers
+// (n = 8, posted, F = 3, 65,000 pairs 103 us, 123 in one)
+template <int n, bool DF, bool FIELD>
 __global__ void __launch_bounds__(128) k_eval_pairs(EvalPairsArgs A, BasisTab tab)
 {
     constexpr int n3 = n * n * n;
-    const int nf = A.ev.F / (int)gridDim.y;
+    const int nf = FIELD ? A.ev.F / (int)gridDim.y : 0;   // (1; a constant 1 gives slower code)
     const int64_t f0 = (int64_t)blockIdx.y * nf;
     int64_t s0 = 0, s1;
     if (A.s_lo) {
@@ -558,10 +592,13 @@ __global__ void __launch_bounds__(128) k_eval_pairs(EvalPairsArgs A, BasisTab ta
         const int e = A.pair_elem[q] - A.ebase;
         const int64_t w = A.walk ? s : q;
         const double r0 = A.prst[w], r1 = A.prst[A.cap + w], r2 = A.prst[2 * A.cap + w];
-        if (DF)
-            eval_point_df<n>(A.ev.fdf + f0 * A.E * n3, A.E, nf, e, r0, r1, r2, tab, A.ev.out + f0 * A.P, A.P, p);
-        else
-            eval_point_f64<n>(A.ev.f64 + f0 * A.E * n3, A.E, nf, e, r0, r1, r2, tab, A.ev.out + f0 * A.P, A.P, p);
+        if constexpr (FIELD) {
+            if (DF) eval_point_df<n>(A.ev.fdf + f0 * A.E * n3, A.E, nf, e, r0, r1, r2, tab, A.ev.out + f0 * A.P, A.P, p);
+            else eval_point_f64<n>(A.ev.f64 + f0 * A.E * n3, A.E, nf, e, r0, r1, r2, tab, A.ev.out + f0 * A.P, A.P, p);
+        } else {
+            if (DF) eval_point_df<n>(A.ev.fdf, A.E, A.ev.F, e, r0, r1, r2, tab, A.ev.out, A.P, p);
+            else eval_point_f64<n>(A.ev.f64, A.E, A.ev.F, e, r0, r1, r2, tab, A.ev.out, A.P, p);
+        }
     }
 }
 
@@ -653,18 +690,21 @@ cudaError_t launch_eval_pairs(int n, int64_t E, int64_t P, const int32_t* dcount
     const bool df = ev.fdf != nullptr;
     const int64_t stage_bytes = (int64_t)ev.F * n * n * n * (int64_t)sizeof(float2);
     const bool staged = df && ev.staged && stage_bytes <= kStageMaxBytes;
-    // (the staging that a caller asked for comes first)
-    const bool planes = !s_lo && !staged && P <= kPlanePairs;
-    const bool split = !s_lo && !staged && P <= kSplitPairs && n >= kSplitMinN && ev.F <= kSplitFields;
-    const dim3 grid2(grid, split ? ev.F : 1);
+    // (batches: one thread per pair; the staging that a caller asked for comes first)
+    const PairForm form = s_lo || staged ? PAIR_THREAD : pair_form(n, P, ev.F, df);
+    const bool planes = form == PAIR_PLANES;
+    const bool field = form == PAIR_FIELD;
+    const dim3 grid2(grid, ev.F);
     switch (n) {
 #define FP_CASE(NN)                                                                       \
     case NN:                                                                              \
         if (planes && df) k_eval_pairs_planes<NN, PlanesDf><<<grid * kPlaneGroup<NN>, 128, 0, s>>>(a, ev.fdf, tab); \
         else if (planes) k_eval_pairs_planes<NN, PlanesF64><<<grid * kPlaneGroup<NN>, 128, 0, s>>>(a, ev.f64, tab); \
         else if (staged) k_eval_pairs_staged<NN><<<grid, kStageTile, stage_bytes, s>>>(a, tab); \
-        else if (df) k_eval_pairs<NN, true><<<grid2, 128, 0, s>>>(a, tab);                \
-        else k_eval_pairs<NN, false><<<grid2, 128, 0, s>>>(a, tab);                       \
+        else if (field && df) k_eval_pairs<NN, true, (NN >= kFieldMinN)><<<grid2, 128, 0, s>>>(a, tab); \
+        else if (field) k_eval_pairs<NN, false, (NN >= kFieldMinN)><<<grid2, 128, 0, s>>>(a, tab); \
+        else if (df) k_eval_pairs<NN, true, false><<<grid, 128, 0, s>>>(a, tab);          \
+        else k_eval_pairs<NN, false, false><<<grid, 128, 0, s>>>(a, tab);                 \
         break;
         FP_CASE(2) FP_CASE(3) FP_CASE(4) FP_CASE(5) FP_CASE(6) FP_CASE(7) FP_CASE(8) FP_CASE(9)
         FP_CASE(10) FP_CASE(11) FP_CASE(12) FP_CASE(13) FP_CASE(14) FP_CASE(15) FP_CASE(16)

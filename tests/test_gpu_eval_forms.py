@@ -1,5 +1,6 @@
 """Which kernel an evaluation runs (the forms give the same bits): staging in
-shared memory whenever it is asked for."""
+shared memory whenever it is asked for, planes only where they are the faster
+form, and every form of a fused evaluation against the separate one."""
 import numpy as np
 import pytest
 import torch
@@ -33,3 +34,27 @@ def test_staging_is_done_when_asked_for(N, F, P):
     assert has(names, "k_eval_pairs_staged")
     for a, b in zip(plain, staged):
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("N,F,P,planes", [(7, 2, 5000, True), (7, 12, 15000, None), (9, 2, 5000, True), (9, 3, 5000, False),
+                                          (12, 6, 2000, None), (5, 3, 20000, True), (5, 3, 30000, False), (7, 3, 45000, False)])
+def test_fused_forms(N, F, P, planes, prec):
+    fg, h, pts, kw = setup(N, F, P, prec)
+    out, names = kernel_names(lambda: fg.fp_find_eval(h, pts, **kw))
+    if planes is None:
+        planes = prec == 0
+    assert has(names, "k_eval_pairs_planes") == planes
+    sep = fg.fp_eval_df(h, kw["posted"], out[0], out[2], out[3]) if prec else fg.fp_eval(h, out[0], out[2], out[3], kw["fields"])
+    np.testing.assert_array_equal(out[5].cpu().numpy(), sep.cpu().numpy())
+
+
+@pytest.mark.parametrize("F,P,planes", [(1, 10000, True), (1, 10001, False), (3, 3000, True), (4, 1000, False)])
+def test_posted_points(F, P, planes):
+    fg, h, pts, kw = setup(7, F, P, 1)
+    out = fg.fp_find(h, pts)
+    q = fg.Points(h, P)
+    q.set(out[0], out[2], out[3])
+    v, names = kernel_names(lambda: q.eval(kw["posted"]))
+    assert has(names, "k_eval_planes") == planes and has(names, "k_eval_points_df") != planes
+    np.testing.assert_array_equal(v.cpu().numpy(), fg.fp_eval_df(h, kw["posted"], out[0], out[2], out[3]).cpu().numpy())
