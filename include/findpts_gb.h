@@ -568,6 +568,20 @@ fp_status fp_newton_paths(fp_handle *h, int64_t *counts);
  * Errors: FP_ERR_NOT_SETUP, FP_ERR_INVALID_ARG (out of range). */
 fp_status fp_set_mixed_refine(fp_handle *h, int max_residuals);
 
+/* Node digits of a hexahedral mesh (the layout that the tensor-core Newton
+ * kernels read; FP64 form of orders 3-9, mixed form of orders 4, 6-9): with
+ * keep != 0 they are stored, N = 7: 18 kB (FP64 form) or 34 kB (mixed form) an
+ * element; with 0 they are released and made from the coordinates in every
+ * find, which takes longer (FP64 form 1.2 to 2.5 times, mixed form 1.7 to 12
+ * times, most with many points an element) and gives the same results bit for
+ * bit.  After fp_setup they are stored if they take at most half of the free
+ * device memory.  Batches copy the state their handles have when they are created;
+ * other handles ignore the call.  Waits for the device; not to be called while
+ * a graph that was captured from this handle is still to be launched.
+ * Errors: FP_ERR_NOT_SETUP, FP_ERR_OOM (keep != 0; the handle stays usable),
+ * FP_ERR_CUDA. */
+fp_status fp_set_node_digits(fp_handle *h, int keep);
+
 /* Fused evaluation of posted (double-float) fields (Sec. 2.1 findpts_eval):
  * with enable != 0, each block copies the fields of every element its 128
  * sorted (point, element) pairs touch into shared memory once and reads the

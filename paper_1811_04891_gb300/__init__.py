@@ -161,6 +161,8 @@ def _load():
     L.fp_profile.restype = ci
     L.fp_set_mixed_refine.argtypes = [vp, ci]
     L.fp_set_mixed_refine.restype = ci
+    L.fp_set_node_digits.argtypes = [vp, ci]
+    L.fp_set_node_digits.restype = ci
     L.fp_set_eval_staging.argtypes = [vp, ci]
     L.fp_set_eval_staging.restype = ci
     L.fp_profile_read.argtypes = [vp, ci, ctypes.POINTER(ctypes.c_double), ctypes.POINTER(i64)]
@@ -782,6 +784,12 @@ PROF_KINDS = {"screen": 0, "sort": 1, "newton": 2, "rank": 3, "eval": 4}
 
 def fp_profile(h: Handle, enable: bool = True):
     _check(lib().fp_profile(h.ptr, int(bool(enable))), h.ptr)
+
+
+def fp_set_node_digits(h: Handle, keep: bool = True):
+    """Store the node digits that the tensor-core Newton kernels read, or
+    release them (finds make them on the fly: slower, same results)."""
+    _check(lib().fp_set_node_digits(h.ptr, int(bool(keep))), h.ptr)
 
 
 def fp_set_eval_staging(h: Handle, enable: bool = True):

@@ -359,8 +359,15 @@ extern "C" fp_status fp_batch_create(fp_batch** out, int ninst, fp_handle* const
         if (e == cudaSuccess && b->mixed) e = alloc(&g.coords32, 3 * g.E * n3);
         const bool lo = b->mixed && !is_tile_order(g.n, true);
         if (e == cudaSuccess && lo) e = alloc(&g.coords32lo, 3 * g.E * n3);
-        const int64_t db = tile_digits_bytes(g.n, b->mixed);
-        if (e == cudaSuccess && db > 0) e = alloc(&g.digits, g.E * db);
+        // digits: where every handle has them and they fit (else made where they are used)
+        int64_t db = tile_digits_bytes(g.n, b->mixed);
+        for (int i : g.inst)
+            if (!handles[i]->digits) db = 0;
+        if (e == cudaSuccess && db > 0 && alloc(&g.digits, g.E * db) != cudaSuccess) {
+            if ((e = cudaGetLastError()) == cudaErrorMemoryAllocation) e = cudaSuccess;
+            g.digits = nullptr;
+            db = 0;
+        }
         if (e == cudaSuccess) e = alloc(&g.boxes, g.E);
         if (e == cudaSuccess && multi) e = alloc(&g.dist, g.E * n3);
         if (e == cudaSuccess && F > 0) e = alloc(&g.fields, (int64_t)F * g.E * n3);
@@ -468,9 +475,18 @@ extern "C" fp_status fp_batch_create(fp_batch** out, int ninst, fp_handle* const
         if (e == cudaSuccess) e = alloc(&b->prst, 3 * b->cap);
         bool tile = false;
         for (auto& g : b->groups) tile = tile || is_tile_order(g.n, b->mixed);
-        if (e == cudaSuccess && (tile || !b->mixed)) e = alloc(&b->pstate, b->cap);
-        if (e == cudaSuccess && tile) e = alloc(&b->pause_list, b->cap);
-        if (e == cudaSuccess && tile && b->mixed) e = alloc(&b->jst, 9 * b->cap);
+        if (e == cudaSuccess && !b->mixed) e = alloc(&b->pstate, b->cap);
+        // tile groups do without these where they don't fit (one Newton launch, the same results)
+        if (e == cudaSuccess && tile && ((b->mixed && alloc(&b->pstate, b->cap) != cudaSuccess) ||
+                                         alloc(&b->pause_list, b->cap) != cudaSuccess ||
+                                         (b->mixed && alloc(&b->jst, 9 * b->cap) != cudaSuccess))) {
+            if ((e = cudaGetLastError()) == cudaErrorMemoryAllocation) e = cudaSuccess;
+            if (b->mixed) release(b->pstate);
+            release(b->pause_list); release(b->jst);
+            b->pause_list = nullptr;
+            b->jst = nullptr;
+            if (b->mixed) b->pstate = nullptr;
+        }
         if (e == cudaSuccess) e = alloc(&b->inv, b->cap);
         if (e == cudaSuccess) e = alloc(&b->band, 3);
         if (e == cudaSuccess) e = cudaMemset(b->band, 0, 3 * sizeof(unsigned long long));

@@ -30,7 +30,9 @@ struct fp_handle {
     double* coords = nullptr;      // [3][E][n3]
     float* coords32 = nullptr;     // [3][E][n3] element-local FP32 (mixed form)
     float* coords32lo = nullptr;   // [3][E][n3] low parts: (x - c) - coords32 (mixed form)
-    unsigned char* digits = nullptr;   // [E][tile_digits_bytes(n)] node digits (hexahedra, orders of the tile kernels)
+    unsigned char* digits = nullptr;   // [E][tile_digits_bytes(n)] node digits (hexahedra, orders of the tile
+                                   //   kernels); null: made from the coordinates where they are used
+    bool keep_digits = true;       // lay them out at the next (re)build
     int32_t* sub = nullptr;        // [E]
     double* dist = nullptr;        // [E][n3] or null
     fpg::ElemBox* boxes = nullptr;      // [E]

@@ -198,6 +198,8 @@ void release(fp_handle* h)
     h->h_total = nullptr;
 }
 
+bool has_tiles(const fp_handle* h) { return h->dim == 3 && is_tile_order(h->n, h->opts.precision == FP_PREC_MIXED); }
+
 // whether finds on this handle pause solves after a first Newton pass (the
 // FP64 form, and both forms with tile kernels); bytes per pair that takes
 bool keeps_state(const fp_handle* h)
@@ -207,8 +209,37 @@ bool keeps_state(const fp_handle* h)
 
 int64_t pause_bytes(const fp_handle* h)
 {
-    const bool tile = h->dim == 3 && is_tile_order(h->n, h->opts.precision == FP_PREC_MIXED);
+    const bool tile = has_tiles(h);
     return (keeps_state(h) ? 16 : 0) + (tile ? 4 : 0) + (tile && h->opts.precision == FP_PREC_MIXED ? 36 : 0);
+}
+
+// The buffers a find of a tile order can do without (it then runs its Newton
+// stage in one launch, with the same results): left out where they don't fit.
+// (pstate of the other orders' FP64 form stays required.)
+template <typename E>
+bool alloc_pause(const fp_handle* h, int64_t cap, double2** pstate, E** list, float** jst)
+{
+    if (!has_tiles(h)) return true;
+    if (dalloc(pstate, cap) == cudaSuccess && dalloc(list, cap) == cudaSuccess &&
+        (h->opts.precision != FP_PREC_MIXED || dalloc(jst, 9 * cap) == cudaSuccess))
+        return true;
+    dfree(*pstate); dfree(*list); dfree(*jst);
+    return cudaGetLastError() == cudaErrorMemoryAllocation;   // (and cleared)
+}
+
+// Stored node digits take 0.75 (FP64 form) to 1.4 times (mixed form, N = 7)
+// the mesh's other resident memory: laid out when they take at most half of
+// what is free (at 270 GB and N = 7: 7.3 and 4 million elements).
+void try_digits(fp_handle* h)
+{
+    if (h->digits || !h->keep_digits) return;
+    const size_t want = (size_t)h->E * tile_digits_bytes(h->n, h->opts.precision == FP_PREC_MIXED);
+    size_t free = 0, total = 0;
+    if (cudaMemGetInfo(&free, &total) != cudaSuccess || want > free / 2 || dalloc(&h->digits, want) != cudaSuccess) {
+        (void)cudaGetLastError();
+        h->digits = nullptr;
+        h->keep_digits = false;
+    }
 }
 
 fp_status grow_points(fp_handle* h, int64_t P)
@@ -235,16 +266,14 @@ fp_status grow_pairs(fp_handle* h, int64_t np)
     cudaDeviceSynchronize();
     dfree(h->pair_elem); dfree(h->pair_pt); dfree(h->order); dfree(h->pres); dfree(h->prst); dfree(h->pstate);
     dfree(h->inv); dfree(h->pause_list); dfree(h->jst);
-    const bool tile = h->dim == 3 && is_tile_order(h->n, h->opts.precision == FP_PREC_MIXED), two_pass = keeps_state(h);
-    const bool mixed = h->opts.precision == FP_PREC_MIXED;
+    const bool two_pass = keeps_state(h) && !has_tiles(h);
     cudaError_t e;
     if ((e = dalloc(&h->pair_elem, cap)) != cudaSuccess || (e = dalloc(&h->pair_pt, cap)) != cudaSuccess ||
         (e = dalloc(&h->order, cap)) != cudaSuccess || (e = dalloc(&h->pres, cap)) != cudaSuccess ||
         (e = dalloc(&h->prst, 3 * cap)) != cudaSuccess ||
         (h->dim == 3 && (e = dalloc(&h->inv, cap)) != cudaSuccess) ||
         (two_pass && (e = dalloc(&h->pstate, cap)) != cudaSuccess) ||
-        (tile && (e = dalloc(&h->pause_list, cap)) != cudaSuccess) ||
-        (tile && mixed && (e = dalloc(&h->jst, 9 * cap)) != cudaSuccess)) {
+        (!alloc_pause(h, cap, &h->pstate, &h->pause_list, &h->jst) && (e = cudaErrorUnknown) != cudaSuccess)) {
         h->cap_pairs = 0;
         return cuda_fail(h, e, "workspace (pairs)");
     }
@@ -423,8 +452,8 @@ fp_status build_geometry(fp_handle* h, cudaStream_t s, bool default_dist)
 
     // node digits of the tile kernels, with each element's scale and affine deviation
     const bool mixed = o.precision == FP_PREC_MIXED;
-    if (h->dim == 3 && is_tile_order(n, mixed)) {
-        if (!h->digits) GK(dalloc(&h->digits, (size_t)E * tile_digits_bytes(n, mixed)), "alloc digits");
+    if (has_tiles(h)) {
+        try_digits(h);
         GK(launch_digits(n, mixed, E, h->coords, h->boxes, h->digits, h->tab, s), "digits");
     }
 
@@ -829,9 +858,8 @@ fp_status fp_workspace_create(const fp_handle* h, int64_t max_points, int64_t ma
         (e = dalloc(&w->order, max_pairs)) != cudaSuccess || (e = dalloc(&w->ecount, h->E)) != cudaSuccess ||
         (e = dalloc(&w->estart, h->E + 1)) != cudaSuccess || (e = dalloc(&w->pres, max_pairs)) != cudaSuccess ||
         (e = dalloc(&w->prst, 3 * max_pairs)) != cudaSuccess || (e = dalloc(&w->inv, max_pairs)) != cudaSuccess ||
-        (keeps_state(h) && (e = dalloc(&w->pstate, max_pairs)) != cudaSuccess) ||
-        (is_tile_order(h->n, h->opts.precision == FP_PREC_MIXED) && (e = dalloc(&w->pause_list, max_pairs)) != cudaSuccess) ||
-        (is_tile_order(h->n, h->opts.precision == FP_PREC_MIXED) && h->opts.precision == FP_PREC_MIXED && (e = dalloc(&w->jst, 9 * max_pairs)) != cudaSuccess)) {
+        (keeps_state(h) && !has_tiles(h) && (e = dalloc(&w->pstate, max_pairs)) != cudaSuccess) ||
+        (!alloc_pause(h, max_pairs, &w->pstate, &w->pause_list, &w->jst) && (e = cudaErrorUnknown) != cudaSuccess)) {
         ws_release(w);
         delete w;
         return e == cudaErrorMemoryAllocation ? FP_ERR_OOM : FP_ERR_CUDA;
@@ -1139,6 +1167,34 @@ fp_status fp_set_eval_staging(fp_handle* h, int enable)
     if (!fp_live(h)) return FP_ERR_NOT_SETUP;
     h->stage_eval = enable != 0;
     return FP_OK;
+}
+
+fp_status fp_set_node_digits(fp_handle* h, int keep)
+{
+    if (!fp_live(h)) return FP_ERR_NOT_SETUP;
+    if (!has_tiles(h) || (keep != 0) == (h->digits != nullptr)) {
+        h->keep_digits = keep != 0;
+        return FP_OK;
+    }
+    cudaError_t e = cudaDeviceSynchronize();             // no find is reading them
+    if (e != cudaSuccess) return cuda_fail(h, e, "fp_set_node_digits");
+    h->keep_digits = keep != 0;
+    if (!keep) {
+        dfree(h->digits);
+        return FP_OK;
+    }
+    const bool mixed = h->opts.precision == FP_PREC_MIXED;
+    e = dalloc(&h->digits, (size_t)h->E * tile_digits_bytes(h->n, mixed));
+    if (e == cudaSuccess) {
+        e = launch_digits(h->n, mixed, h->E, h->coords, h->boxes, h->digits, h->tab, nullptr);
+        if (e == cudaSuccess) e = cudaDeviceSynchronize();
+    }
+    if (e == cudaSuccess) return FP_OK;
+    if (e == cudaErrorMemoryAllocation) (void)cudaGetLastError();
+    dfree(h->digits);
+    h->digits = nullptr;
+    h->keep_digits = false;
+    return cuda_fail(h, e, "fp_set_node_digits");
 }
 
 fp_status fp_set_mixed_refine(fp_handle* h, int max_residuals)

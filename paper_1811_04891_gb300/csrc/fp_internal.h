@@ -122,7 +122,7 @@ struct FindArgs {
     uint32_t* smask = nullptr;    // [P] screen: candidates that passed the count pass, by bit of the
                                   //   cell list (bit 31: list too long, test again); null = test again
     int batch = 0;                // 1: a batch group (its own FP64 first-pass budget)
-    const unsigned char* digits = nullptr;   // the elements' node digits (orders of the tile kernels)
+    const unsigned char* digits = nullptr;   // the elements' node digits (orders of the tile kernels; null: made on the fly)
     int32_t* pause_list = nullptr;           // [cap] tile kernels: paused solves (with pstate); null: one pass
     float* jst = nullptr;                    // [9][cap] mixed form: Jacobians kept between its two launches
     int32_t* pause_count = nullptr;          // batch groups: their number (otherwise the second scan scratch word)
@@ -130,7 +130,8 @@ struct FindArgs {
 
 // Tensor-core tile kernels (fp_tile.cuh) of the Newton stage: their orders,
 // the bytes of an element's node digits (0 for other orders) and the kernel
-// that lays them out (also boxes[].scale, cscale, jscale and dev).
+// that lays them out (also boxes[].scale, cscale, jscale and dev; dig null:
+// these alone).
 //
 // The order decides alone, never the number of points, so that every entry
 // point gives a pair the same bits.  Lower orders have too little to contract,

@@ -29,6 +29,8 @@ namespace fpg {
 cudaError_t FP_CAT(newton_tile_mixed_, FP_N)(const FindArgs& a, const NewtonArgs& na, int64_t npairs, const BasisTab& tab,
                                              int block, unsigned grid, cudaStream_t s);
 int FP_CAT(tile_fit_mixed_, FP_N)(int block);
+cudaError_t FP_CAT(digits_mixed_, FP_N)(int64_t E, const double* coords, ElemBox* boxes, unsigned char* dig,
+                                        const BasisTab& tab, cudaStream_t s);
 
 // ---------------------------------------------------------------------------
 // Newton kernels, one thread per pair (the solver is in fp_newton.cuh)
@@ -542,8 +544,9 @@ template <int n, bool MIXED>
 static cudaError_t digits_if(int64_t E, const double* coords, ElemBox* boxes, unsigned char* dig, const BasisTab& tab,
                              cudaStream_t s)
 {
-    if constexpr (is_tile_order(n, MIXED)) return digits_form<n, MIXED>(E, coords, boxes, dig, tab, s);
-    else return cudaErrorInvalidValue;
+    if constexpr (!is_tile_order(n, MIXED)) return cudaErrorInvalidValue;
+    else if constexpr (MIXED) return FP_CAT(digits_mixed_, FP_N)(E, coords, boxes, dig, tab, s);
+    else return digits_form<n, false>(E, coords, boxes, dig, tab, s);
 }
 
 template <int n, bool MIXED>

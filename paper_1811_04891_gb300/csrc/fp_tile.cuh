@@ -172,18 +172,31 @@ __device__ __forceinline__ int2 fix60(double h)
     return make_int2(__double2loint(p), __double2loint(q));
 }
 
-// the product of two of them in units of 2^-60 (y y' left out), by integer
-// multiply-adds: the FP64 pipe, with 3 operations a product, was what bounded
-// the kernel (2.0e6 points, N = 7, whole find and evaluation: 26.1 ms).  The
-// bias makes digit s the bits 51 - 10 s and up, plus 512, rounded to 2^-59.
+// makes digit s of a fixed-point value of unit 2^-60 the bits 51 - 10 s and up,
+// plus 512, rounded to 2^-59
+constexpr int64_t kBias60 = 512ll * ((1ll << 51) + (1ll << 41) + (1ll << 31) + (1ll << 21) + (1ll << 11) + (1ll << 1)) + 1;
+
+// the product of two basis values in units of 2^-60 (y y' left out) plus the
+// bias, by integer multiply-adds: the FP64 pipe, with 3 operations a product,
+// was what bounded the kernel (2.0e6 points, N = 7, whole find and evaluation:
+// 26.1 ms)
 __device__ __forceinline__ uint64_t product60(int2 a, int2 b)
 {
-    constexpr int64_t bias = 512ll * ((1ll << 51) + (1ll << 41) + (1ll << 31) + (1ll << 21) + (1ll << 11) + (1ll << 1)) + 1;
     const int64_t low = (int64_t)a.x * b.y + ((int64_t)a.y * b.x + (1 << 29));
-    return (uint64_t)(((int64_t)a.x * b.x + bias) + (low >> 30));
+    return (uint64_t)(((int64_t)a.x * b.x + kBias60) + (low >> 30));
 }
 
-// three digits of two products, as FP16 pairs: f is the FP16 number 1024 + f
+// v 2^-e in units of 2^-60 (|v| < 2^(e-1)) plus the bias
+__device__ __forceinline__ uint64_t fixed60(double v, int e)
+{
+    const int64_t b = __double_as_longlong(v);
+    const int x = (int)((b >> 52) & 0x7ff), sh = 1015 + e - max(x, 1);      // right shift
+    const int64_t m = (b & 0xfffffffffffffll) | (x ? 1ll << 52 : 0);
+    const int64_t k = sh <= 0 ? m << -sh : sh > 54 ? 0 : (m + (1ll << (sh - 1))) >> sh;
+    return (uint64_t)((b < 0 ? -k : k) + kBias60);
+}
+
+// three digits of two values, as FP16 pairs: f is the FP16 number 1024 + f
 // (bits 0x6400 + f) minus 1536; the first digit of all reaches 512 (11 bits)
 template <bool FIRST>
 __device__ __forceinline__ void fields3(uint32_t u, uint32_t w, uint32_t* o)
@@ -197,12 +210,16 @@ __device__ __forceinline__ void fields3(uint32_t u, uint32_t w, uint32_t* o)
     }
 }
 
-// 6 digits
-__device__ __forceinline__ void digits2(int2 a0, int2 b0, int2 a1, int2 b1, uint32_t (&o)[6])
+// the 6 digits of two biased fixed-point values
+__device__ __forceinline__ void fields6(uint64_t u, uint64_t w, uint32_t (&o)[6])
 {
-    const uint64_t u = product60(a0, b0), w = product60(a1, b1);
     fields3<true>((uint32_t)(u >> 31), (uint32_t)(w >> 31), o);
     fields3<false>((uint32_t)(u >> 1), (uint32_t)(w >> 1), o + 3);
+}
+
+__device__ __forceinline__ void digits2(int2 a0, int2 b0, int2 a1, int2 b1, uint32_t (&o)[6])
+{
+    fields6(product60(a0, b0), product60(a1, b1), o);
 }
 
 // ---- the element's nodes as digits, in B-fragment order ----
@@ -273,6 +290,87 @@ struct RightFrag {
     }
 };
 
+// ---- fragments of an element without stored digits ----
+// The digits that k_digits lays out, made from the coordinates where they are
+// used (with the scales it left in boxes): the same bits for no memory.  m: 0
+// the nodes, 1 and 2 (mixed form) the nodal values of dx/dr and dx/ds, whose
+// rows of n products are most of the cost.  A find, stored / made here, us:
+// N = 7, 4,096 elements, FP64 form 1,000 points 341/439, 400,000 2768/4413;
+// mixed form 157/275, 890/7330; N = 9 mixed 1,820/22,966.
+struct NodeSource {
+    const double* coords;
+    const float* coords32;
+    const ElemBox* boxes;
+    int64_t E;
+    const float* der;                  // der[i n + u] = h_u'(xi_i) (mixed form)
+};
+
+__device__ __forceinline__ int exp_of(double p) { return ((__double2hiint(p) >> 20) & 0x7ff) - 1023; }
+__device__ __forceinline__ int exp_of(float p) { return ((__float_as_int(p) >> 23) & 0xff) - 127; }
+
+// one of the nodal values of dx/dr (st = 1) or dx/ds (st = n): the row through
+// v times the derivatives of row `at`
+template <int n>
+__device__ __forceinline__ float nodal_derivative(const float* der, const float* v, int at, int st)
+{
+    float w = 0.0f;
+#pragma unroll
+    for (int u = 0; u < n; ++u) w = fmaf(der[at * n + u], v[u * st], w);
+    return w;
+}
+
+// rows of the table by the block's first n threads
+template <int n>
+__device__ __forceinline__ void derivative_table(const BasisTab& tab, float* der)
+{
+    if (threadIdx.x < n) {
+        float h[n], d[n];
+        lagrange_hd<n, float>(tab.xif, tab.cif, tab.xif[threadIdx.x], h, d);
+#pragma unroll
+        for (int m = 0; m < n; ++m) der[threadIdx.x * n + m] = d[m];
+    }
+}
+
+template <int n, int S>
+__device__ __forceinline__ void make_frag(const NodeSource& N, int el, int kc, int t, int m, RightFrag<S>& R)
+{
+    constexpr int n2 = n * n, n3 = n2 * n;
+    const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
+    const int col = 8 * t + g, a = col < n ? 0 : col < 2 * n ? 1 : 2, k = col - a * n;
+    const ElemBox& bx = N.boxes[el];
+    const int64_t plane = ((int64_t)a * N.E + el) * n3 + n2 * k;
+#pragma unroll
+    for (int hf = 0; hf < 2; ++hf) {
+        const int kap = 16 * kc + 8 * hf + 2 * q;
+        if (m == 0) {
+            uint64_t w[2];
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const bool in = kap + u < n2 && col < 3 * n;
+                w[u] = fixed60(in ? __ldg(N.coords + plane + kap + u) - bx.c[a] : 0.0, exp_of(bx.scale) + exp_of(bx.cscale[a]));
+            }
+            uint32_t d[6];
+            fields6(w[0], w[1], d);
+#pragma unroll
+            for (int s = 0; s < S; ++s) R.b[s][hf] = d[s];
+        } else if constexpr (S == 3) {
+            float v[2];
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int x = kap + u, at = m == 1 ? x % n : x / n, st = m == 1 ? 1 : n;
+                const bool in = x < n2 && col < 3 * n;
+                v[u] = in ? ldexpf(nodal_derivative<n>(N.der, N.coords32 + plane + x - at * st, at, st),
+                                   -(exp_of(bx.scale) + exp_of(bx.jscale[m - 1][a])))
+                          : 0.0f;
+            }
+            uint32_t d[3];
+            digits2(v[0], 1.0f, v[1], 1.0f, d);
+#pragma unroll
+            for (int s = 0; s < S; ++s) R.b[s][hf] = d[s];
+        }
+    }
+}
+
 // acc[o][t] += the order-o products of S left digits and the S right digits of
 // tile t; FINE: order S joins the sums of order S - 1, its right digits scaled
 // by 2^-10
@@ -295,19 +393,16 @@ __device__ __forceinline__ void mma_digits(const uint32_t (&a)[S][4], const Righ
 }
 
 // acc = the digit products of a 16-row tile over all k16 steps.  left(kc, a)
-// gives the tile's digits; base + el * ebytes are an element's fragments (sb
-// digits stored).  One element among the rows: the next step's fragments are
-// fetched while the current ones are multiplied (three digits: they fit the
-// registers).  Several: each element's rows in turn, the others masked to
-// zero.
-template <int n, int S, int O, bool FINE, typename Left>
-__device__ __forceinline__ void tile_gemm(Left&& left, const unsigned char* __restrict__ base, int sb, int64_t ebytes,
-                                          uint32_t heads, uint32_t need, int e, int mt,
+// gives the tile's digits, right(el, kc, t, R) an element's fragments.  One
+// element among the rows: the next step's fragments are fetched while the
+// current ones are multiplied (three digits: they fit the registers).
+// Several: each element's rows in turn, the others masked to zero.
+template <int n, int S, int O, bool FINE, typename Left, typename Right>
+__device__ __forceinline__ void tile_gemm(Left&& left, Right&& right, uint32_t heads, uint32_t need, int e, int mt,
                                           float (&acc)[O][TileDim<n>::NT][4])
 {
     using D = TileDim<n>;
     const int lane = threadIdx.x & 31, g = lane >> 2;
-    const int step = D::NT * FragBytes<1>::v * sb;
 #pragma unroll
     for (int o = 0; o < O; ++o)
 #pragma unroll
@@ -323,21 +418,22 @@ __device__ __forceinline__ void tile_gemm(Left&& left, const unsigned char* __re
         if ((need >> h) & ((1u << (nx - h)) - 1u)) hs |= 1u << h;
     }
     if (!hs) return;
-    auto frag = [&](int h, int kc) { return base + (int64_t)__shfl_sync(kFull, e, 16 * mt + h) * ebytes + kc * step; };
+    auto elem = [&](int h) { return __shfl_sync(kFull, e, 16 * mt + h); };
     RightFrag<S> next[S == 3 ? D::NT : 1];
-    auto fetch = [&](const unsigned char* F) {
+    auto fetch = [&](int h, int kc) {
+        const int el = elem(h);
 #pragma unroll
-        for (int t = 0; t < D::NT; ++t) next[t].load(F + t * FragBytes<1>::v * sb, sb);
+        for (int t = 0; t < D::NT; ++t) right(el, kc, t, next[t]);
     };
     if constexpr (S == 3) {
-        fetch(frag(__ffs(hs) - 1, 0));
+        fetch(__ffs(hs) - 1, 0);
         if (heads == 1u) {
 #pragma unroll 1
             for (int kc = 0; kc < D::KC; ++kc) {
                 RightFrag<S> R[D::NT];
 #pragma unroll
                 for (int t = 0; t < D::NT; ++t) R[t] = next[t];
-                if (kc + 1 < D::KC) fetch(frag(0, kc + 1));
+                if (kc + 1 < D::KC) fetch(0, kc + 1);
                 uint32_t a[S][4];
                 left(kc, a);
 #pragma unroll
@@ -370,15 +466,15 @@ __device__ __forceinline__ void tile_gemm(Left&& left, const unsigned char* __re
                 RightFrag<S> R[D::NT];
 #pragma unroll
                 for (int t = 0; t < D::NT; ++t) R[t] = next[t];
-                if (hm || kc + 1 < D::KC) fetch(frag(__ffs(hm ? hm : hs) - 1, hm ? kc : kc + 1));
+                if (hm || kc + 1 < D::KC) fetch(__ffs(hm ? hm : hs) - 1, hm ? kc : kc + 1);
 #pragma unroll
                 for (int t = 0; t < D::NT; ++t) mma_digits<n, S, O, FINE>(am, R[t], t, acc);
             } else {
-                const unsigned char* F = frag(h, kc);
+                const int el = elem(h);
 #pragma unroll
                 for (int t = 0; t < D::NT; ++t) {
                     RightFrag<S> R;
-                    R.load(F + t * FragBytes<1>::v * sb, sb);
+                    right(el, kc, t, R);
                     mma_digits<n, S, O, FINE>(am, R, t, acc);
                 }
             }
@@ -421,13 +517,28 @@ __device__ __forceinline__ double column_f64(float a0, float a1, float a2, float
 }
 
 // ---- collective evaluations: lane l holds row l ----
-template <int n>
+template <int n, bool FLY>
 struct TileCtx {
     unsigned char* sm;                 // this warp's shared memory
-    const unsigned char* dig;
+    const unsigned char* dig;          // stored digits
+    NodeSource src;                    // FLY: what they are made from
     uint32_t heads;                    // rows whose element differs from the row before
     int e;                             // the row's element
     const ElemBox* bx;
+
+    // fragment (kc, t) of quantity m (see make_frag): S digits of those stored
+    template <int S, bool MIXED>
+    __device__ __forceinline__ void frag(int el, int kc, int t, int m, RightFrag<S>& R) const
+    {
+        using TB = TileBytes<n, MIXED>;
+        if constexpr (FLY) {
+            make_frag<n, S>(src, el, kc, t, m, R);
+        } else {
+            const int sb = MIXED && m > 0 ? 3 : TB::SX;
+            R.load(dig + (int64_t)el * TB::v + (MIXED && m > 0 ? TB::jac + (m - 1) * TB::one : 0) +
+                       (kc * TileDim<n>::NT + t) * (FragBytes<1>::v * sb), sb);
+        }
+    }
 };
 
 // store one direction's values of this lane's row; the j padding is zero
@@ -493,14 +604,13 @@ template <int n> constexpr int kDerivExp = n <= 4 ? 4 : n <= 5 ? 4 : n <= 6 ? 5 
 
 // map x(r) in the element's frame and scale, and its Jacobian: T = float (to
 // FP32 accuracy, the mixed form's FP32 phase) or double (FP64 form)
-template <int n, typename T>
-__device__ __forceinline__ void tile_fJ(const TileCtx<n>& X, const BasisTab& tab, uint32_t need, bool jac,
+template <int n, typename T, bool FLY>
+__device__ __forceinline__ void tile_fJ(const TileCtx<n, FLY>& X, const BasisTab& tab, uint32_t need, bool jac,
                                         const T (&r)[3], T (&x)[3], T (&J)[9])
 {
     constexpr bool F64 = sizeof(T) == 8;
     using D = TileDim<n>;
     using L = std::conditional_t<F64, Sm64<n>, Sm32<n>>;
-    using TB = TileBytes<n, !F64>;
     constexpr int S = F64 ? 6 : 3, O = S, CS = TileStride<T>::C;
     static_assert((n - 1) * (n - 1) <= 1 << kDerivExp<n>, "derivatives are scaled into [-1,1]");
     const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
@@ -572,8 +682,9 @@ __device__ __forceinline__ void tile_fJ(const TileCtx<n>& X, const BasisTab& tab
                     }
                 }
             };
-            tile_gemm<n, S, O, false>(left, X.dig + (m == 0 || F64 ? 0 : TB::jac + (m - 1) * TB::one), m == 0 || F64 ? TB::SX : 3,
-                               TB::v, hd, nd, X.e, mt, acc);
+            tile_gemm<n, S, O, false>(
+                left, [&](int el, int kc, int t, RightFrag<S>& R) { X.template frag<S, !F64>(el, kc, t, F64 ? 0 : m, R); }, hd,
+                nd, X.e, mt, acc);
             T* C = sm + L::C;
 #pragma unroll
             for (int t = 0; t < D::NT; ++t)
@@ -616,13 +727,12 @@ __device__ __forceinline__ void tile_fJ(const TileCtx<n>& X, const BasisTab& tab
 
 // residual x(r) - x* as double-float, rounded to FP32 (r and xl, the point in
 // the element's frame and scale, as float pairs)
-template <int n>
-__device__ __forceinline__ void tile_f_df(const TileCtx<n>& X, const BasisTab& tab, uint32_t need, const df (&r)[3],
+template <int n, bool FLY>
+__device__ __forceinline__ void tile_f_df(const TileCtx<n, FLY>& X, const BasisTab& tab, uint32_t need, const df (&r)[3],
                                           const df (&xl)[3], float (&f)[3])
 {
     using D = TileDim<n>;
     using L = SmDf<n>;
-    using TB = TileBytes<n, true>;
     constexpr int CS = TileStride<float2>::C, HP = TileStride<float2>::H;
     const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
     float2* sm = reinterpret_cast<float2*>(X.sm);
@@ -643,8 +753,8 @@ __device__ __forceinline__ void tile_f_df(const TileCtx<n>& X, const BasisTab& t
         if (!nd) continue;
         float acc[5][D::NT][4];
         tile_gemm<n, 5, 5, true>(
-            [&](int kc, uint32_t (&a)[5][4]) { tile_left<n, 5, float2>(sm + L::HR, sm + L::HS, kc, mt, a); }, X.dig, 5,
-            TB::v, hd, nd, X.e, mt, acc);
+            [&](int kc, uint32_t (&a)[5][4]) { tile_left<n, 5, float2>(sm + L::HR, sm + L::HS, kc, mt, a); },
+            [&](int el, int kc, int t, RightFrag<5>& R) { X.template frag<5, true>(el, kc, t, 0, R); }, hd, nd, X.e, mt, acc);
         float2* C = sm + L::C;
 #pragma unroll
         for (int t = 0; t < D::NT; ++t)
@@ -867,8 +977,8 @@ __device__ __forceinline__ float inv_norm(const T (&Jd)[9])
 
 // ---- FP64 form: the steps of newton<n, double, true> as a state machine, so
 // that the rows of a warp share their evaluations ----
-template <int n>
-__device__ __forceinline__ void tile_solve_f64(const TileCtx<n>& X, const NewtonArgs& A, const BasisTab& tab, bool active,
+template <int n, bool FLY>
+__device__ __forceinline__ void tile_solve_f64(const TileCtx<n, FLY>& X, const NewtonArgs& A, const BasisTab& tab, bool active,
                                                const double (&xl)[3], double xmax,
                                                double (&r)[3], double& res2, NewtonState& st)
 {
@@ -1002,8 +1112,8 @@ __device__ __forceinline__ void tile_solve_f64(const TileCtx<n>& X, const Newton
 // fate: 0 rejected after it, 1 not converged, 3 left to the full FP64 Newton
 // (refine = 0; res2 < 0 in the last two).  Returns whether the row goes on to
 // the final steps, with r and J from here.
-template <int n>
-__device__ __forceinline__ bool tile_phase32(const TileCtx<n>& X, const NewtonArgs& A, const BasisTab& tab, bool active,
+template <int n, bool FLY>
+__device__ __forceinline__ bool tile_phase32(const TileCtx<n, FLY>& X, const NewtonArgs& A, const BasisTab& tab, bool active,
                                              const double (&xl)[3], double hes, double (&r)[3],
                                              float (&J)[9], double& res2, int& fate, NewtonState& st)
 {
@@ -1129,8 +1239,8 @@ __device__ __forceinline__ bool tile_phase32(const TileCtx<n>& X, const NewtonAr
 // is the code of the latter alone (it fits the instruction cache). ----
 constexpr float kEdge = 0.9999f;
 
-template <int n, bool EDGE>
-__device__ __forceinline__ void tile_final(const TileCtx<n>& X, const NewtonArgs& A, const BasisTab& tab, bool active,
+template <int n, bool EDGE, bool FLY>
+__device__ __forceinline__ void tile_final(const TileCtx<n, FLY>& X, const NewtonArgs& A, const BasisTab& tab, bool active,
                                            const double (&xl)[3], double hes, double (&r)[3], const float (&J)[9],
                                            double& res2, int& fate)
 {
@@ -1288,8 +1398,8 @@ constexpr double kListed = -3.0;       // on the list
 constexpr double kRhoFinal = -1.0;     // pstate.x of a listed pair that ended the FP32 phase
 
 // one warp's rows: pairs s0..s1 of the range (listed: entries of the pause list)
-template <int n, int KIND>
-__device__ __forceinline__ void tile_rows_run(TileCtx<n>& X, const NewtonArgs& A, const BasisTab& tab, bool listed,
+template <int n, int KIND, bool FLY>
+__device__ __forceinline__ void tile_rows_run(TileCtx<n, FLY>& X, const NewtonArgs& A, const BasisTab& tab, bool listed,
                                               int32_t* pl, int32_t* fbl, int64_t fbc, int64_t s0, int64_t s1)
 {
     const int lane = threadIdx.x & 31;
@@ -1416,7 +1526,9 @@ __device__ __forceinline__ void tile_rows_run(TileCtx<n>& X, const NewtonArgs& A
 // 5,550 us so).
 constexpr int kListSpread = 152;
 
-template <int n, int KIND>
+// FLY: no stored digits (A.digits null); the launch's shared memory then ends
+// with the derivative table of the mixed form
+template <int n, int KIND, bool FLY = false>
 __global__ void __launch_bounds__(TileLB<KIND>::threads, TileLB<KIND>::blocks) k_newton_tile(NewtonArgs A, BasisTab tab)
 {
     extern __shared__ uint4 tile_sm[];
@@ -1424,7 +1536,16 @@ __global__ void __launch_bounds__(TileLB<KIND>::threads, TileLB<KIND>::blocks) k
     int32_t* fbl = A.fb_list + (A.s_lo ? R.s0 : 0);
     const int64_t fbc = A.s_lo ? R.s1 - R.s0 : A.fb_cap;
     int32_t* pl = A.pause_list + (A.s_lo ? R.s0 : 0);
-    TileCtx<n> X;
+    TileCtx<n, FLY> X;
+    if constexpr (FLY) {
+        X.src = {A.coords, A.coords32, A.boxes, A.E, nullptr};
+        if constexpr (KIND == TILE_MIXED) {
+            float* der = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(tile_sm) + (blockDim.x >> 5) * TileSmem<n, KIND>::bytes);
+            derivative_table<n>(tab, der);
+            __syncthreads();
+            X.src.der = der;
+        }
+    }
     X.sm = reinterpret_cast<unsigned char*>(tile_sm) + (threadIdx.x >> 5) * TileSmem<n, KIND>::bytes;
     X.dig = A.digits;
     const int nl = KIND == TILE_FINAL ? A.list_blocks : 0;
@@ -1436,7 +1557,7 @@ __global__ void __launch_bounds__(TileLB<KIND>::threads, TileLB<KIND>::blocks) k
     if (KIND == TILE_FINAL && (int)blockIdx.x < nl) {
         const PairRange L{0, (int64_t)*A.pause_count};
         for_each_rows(A, L, rows_of(L.s1, min(nl, kListSpread), 0), false, (int)blockIdx.x, nl, [&](int64_t s0, int64_t s1) {
-            tile_rows_run<n, KIND>(X, A, tab, true, pl, fbl, fbc, s0, s1);
+            tile_rows_run<n, KIND, FLY>(X, A, tab, true, pl, fbl, fbc, s0, s1);
         });
         return;
     }
@@ -1445,7 +1566,7 @@ __global__ void __launch_bounds__(TileLB<KIND>::threads, TileLB<KIND>::blocks) k
     const int nb = (int)gridDim.x - nl;
     for_each_rows(A, L, rows_of(L.s1 - L.s0, nb, listed ? 0 : A.rows), A.queue != nullptr, (int)blockIdx.x - nl, nb,
                   [&](int64_t s0, int64_t s1) {
-                      tile_rows_run<n, KIND>(X, A, tab, KIND == TILE_FP64 && listed, pl, fbl, fbc, s0, s1);
+                      tile_rows_run<n, KIND, FLY>(X, A, tab, KIND == TILE_FP64 && listed, pl, fbl, fbc, s0, s1);
                   });
 }
 
@@ -1485,12 +1606,7 @@ __global__ void __launch_bounds__(128) k_digits(int64_t E, const double* __restr
     __shared__ int4 red[4];
     const int64_t e = blockIdx.x;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (MIXED && threadIdx.x < n) {
-        float h[n], d[n];
-        lagrange_hd<n, float>(tab.xif, tab.cif, tab.xif[threadIdx.x], h, d);
-#pragma unroll
-        for (int m = 0; m < n; ++m) der[threadIdx.x * n + m] = d[m];
-    }
+    if (MIXED) derivative_table<n>(tab, der);
     // the largest of four values over the block, none negative
     auto block_max = [&](int4 v) {
         v = make_int4(__reduce_max_sync(kFull, v.x), __reduce_max_sync(kFull, v.y), __reduce_max_sync(kFull, v.z),
@@ -1535,11 +1651,9 @@ __global__ void __launch_bounds__(128) k_digits(int64_t E, const double* __restr
     const int all = max(most.x, max(most.y, most.z)), ex = all > 0 ? scale_exp(all, -1000) : 0;
     // not below 2^-100 of the largest: within FP32's range
     const int3 ea = make_int3(scale_exp(most.x, ex - 100), scale_exp(most.y, ex - 100), scale_exp(most.z, ex - 100));
-    for (int i = threadIdx.x; i < L::V; i += 128) {       // (the padding too: never read back)
+    for (int i = threadIdx.x; MIXED && i < L::V; i += 128) {   // (the padding too: never read back)
         const int a = i / (n * PL);
-        const double v = V[i] * ldexp(1.0, -(a == 0 ? ea.x : a == 1 ? ea.y : ea.z));
-        V[i] = v;
-        if (MIXED) Vj[i] = (float)v;
+        Vj[i] = (float)(V[i] * ldexp(1.0, -(a == 0 ? ea.x : a == 1 ? ea.y : ea.z)));
     }
     __syncthreads();
     // digits of the values val[], each coordinate divided by its power of two;
@@ -1550,6 +1664,7 @@ __global__ void __launch_bounds__(128) k_digits(int64_t E, const double* __restr
         for (int f = warp; f < D::KC * D::NT; f += 4) {
             const int kc = f / D::NT, t = f % D::NT, g = lane >> 2, q = lane & 3;
             const int col = 8 * t + g;                    // column a n + k is plane a n + k
+            const int x = col < n ? sa.x : col < 2 * n ? sa.y : sa.z;
             RightFrag<SD> R;
 #pragma unroll
             for (int hf = 0; hf < 2; ++hf) {
@@ -1560,31 +1675,23 @@ __global__ void __launch_bounds__(128) k_digits(int64_t E, const double* __restr
                     v[u] = kap < D::n2 && col < 3 * n ? val[col * PL + kap] : TV(0);
                 }
                 uint32_t d[sizeof(TV) == 8 ? 6 : 3];
-                if constexpr (sizeof(TV) == 8) {
-                    const int2 one = make_int2(1 << 30, 0);   // (|v| < 1/2, scaled already)
-                    digits2(fix60(v[0]), one, fix60(v[1]), one, d);
-                } else {
-                    const float ji = ldexpf(1.0f, -(col < n ? sa.x : col < 2 * n ? sa.y : sa.z));
-                    digits2(v[0], ji, v[1], ji, d);
-                }
+                if constexpr (sizeof(TV) == 8) fields6(fixed60(v[0], x), fixed60(v[1], x), d);
+                else digits2(ldexpf(v[0], -x), 1.0f, ldexpf(v[1], -x), 1.0f, d);
 #pragma unroll
                 for (int s = 0; s < SD; ++s) R.b[s][hf] = d[s];
             }
             R.store(out + (int64_t)f * FragBytes<SD>::v);
         }
     };
-    unsigned char* out = dig + e * TB::v;
-    frags(V, make_int3(0, 0, 0), out, std::integral_constant<int, TB::SX>());
+    unsigned char* out = dig + e * TB::v;                 // (dig null: scales and deviation only)
+    if (dig) frags(V, ea, out, std::integral_constant<int, TB::SX>());
     // mixed form: dx/dr and dx/ds, each coordinate with its own power of two
 #pragma unroll 1
     for (int m = 0; MIXED && m < 2; ++m) {
         most = make_int4(0, 0, 0, 0);
         for (int i = threadIdx.x; i < 3 * n3; i += 128) {
             const int c = i / (n * n), q = i % (n * n), at = m == 0 ? q % n : q / n, st = m == 0 ? 1 : n;
-            const float* v = Vj + c * PL + q - at * st;
-            float w = 0.0f;
-#pragma unroll
-            for (int u = 0; u < n; ++u) w += der[at * n + u] * v[u * st];
+            const float w = nodal_derivative<n>(der, Vj + c * PL + q - at * st, at, st);
             W[c * PL + q] = w;
             const int x = expo(w);
             if (i < n3) most.x = max(most.x, x);
@@ -1593,7 +1700,7 @@ __global__ void __launch_bounds__(128) k_digits(int64_t E, const double* __restr
         }
         most = block_max(most);
         const int3 sa = make_int3(scale_exp(most.x, -100), scale_exp(most.y, -100), scale_exp(most.z, -100));
-        frags(W, sa, out + TB::jac + m * TB::one, std::integral_constant<int, 3>());
+        if (dig) frags(W, sa, out + TB::jac + m * TB::one, std::integral_constant<int, 3>());
         if (threadIdx.x == 0) {
             boxes[e].jscale[m][0] = ldexpf(1.0f, sa.x + ea.x - ex);
             boxes[e].jscale[m][1] = ldexpf(1.0f, sa.y + ea.y - ex);

@@ -35,25 +35,28 @@ static cudaError_t raise_smem(std::atomic<uint64_t>& done, K kernel, int bytes)
 }
 
 // (tile kernels: blocks of up to four warps)
-template <int n, int KIND>
+template <int n, int KIND, bool FLY>
+constexpr int tile_smem(int warps) { return warps * TileSmem<n, KIND>::bytes + (FLY && KIND == TILE_MIXED ? n * n * (int)sizeof(float) : 0); }
+
+template <int n, int KIND, bool FLY = false>
 static cudaError_t tile_prepare()
 {
     static std::atomic<uint64_t> done{0};
-    return raise_smem(done, k_newton_tile<n, KIND>, 4 * TileSmem<n, KIND>::bytes);
+    return raise_smem(done, k_newton_tile<n, KIND, FLY>, tile_smem<n, KIND, FLY>(4));
 }
 
 // blocks of `block` threads that fit one SM at once (asked of the runtime once per form and block size)
-template <int n, int KIND>
+template <int n, int KIND, bool FLY = false>
 static int tile_fit(int block)
 {
     static std::atomic<int> known[5];
     std::atomic<int>& slot = known[std::min(block / 32, 4)];
     if (const int v = slot.load()) return v;
     int k = 0;
-    cudaError_t e = tile_prepare<n, KIND>();
+    cudaError_t e = tile_prepare<n, KIND, FLY>();
     if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&k, k_newton_tile<n, KIND>, block,
-                                                          (size_t)(block / 32) * TileSmem<n, KIND>::bytes);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&k, k_newton_tile<n, KIND, FLY>, block,
+                                                          (size_t)tile_smem<n, KIND, FLY>(block / 32));
     if (e != cudaSuccess || k < 1) return 1;
     slot.store(k);
     return k;
@@ -61,19 +64,19 @@ static int tile_fit(int block)
 
 // grid: 0 = one warp per na.rows pairs of npairs; persistent (npairs < 0) =
 // every block that fits the GPU at once; otherwise as given
-template <int n, int KIND>
+template <int n, int KIND, bool FLY = false>
 static cudaError_t launch_tile(const NewtonArgs& na, const BasisTab& tab, int64_t npairs, int block, unsigned grid,
                                cudaStream_t s)
 {
     // whole warps, at most the four of the launch bounds: each has its own shared memory
     if (block < 32 || block > TileLB<KIND>::threads || block % 32 != 0) return cudaErrorInvalidValue;
     const int per = block / 32;
-    const cudaError_t err = tile_prepare<n, KIND>();
+    const cudaError_t err = tile_prepare<n, KIND, FLY>();
     if (err != cudaSuccess) return err;
-    if (npairs < 0) grid = (unsigned)(sm_count() * tile_fit<n, KIND>(block));
+    if (npairs < 0) grid = (unsigned)(sm_count() * tile_fit<n, KIND, FLY>(block));
     else if (grid == 0) grid = (unsigned)std::max<int64_t>(1, (npairs + (int64_t)per * na.rows - 1) / ((int64_t)per * na.rows));
     grid += na.list_blocks;
-    k_newton_tile<n, KIND><<<grid, block, (size_t)per * TileSmem<n, KIND>::bytes, s>>>(na, tab);
+    k_newton_tile<n, KIND, FLY><<<grid, block, (size_t)tile_smem<n, KIND, FLY>(per), s>>>(na, tab);
     count_launch();
     return cudaGetLastError();
 }
@@ -140,7 +143,7 @@ static cudaError_t newton_tile(const FindArgs& a, NewtonArgs na, int64_t npairs,
     const bool fixed = a.persistent_blocks > 0 || a.queue;
     int64_t launch = npairs;                         // < 0: a persistent grid
     if (!fixed) {
-        na.rows = tile_rows(npairs, tblock / 32 * tile_fit<n, KIND>(tblock));
+        na.rows = tile_rows(npairs, tblock / 32 * (na.digits ? tile_fit<n, KIND>(tblock) : tile_fit<n, KIND, true>(tblock)));
         tblock = spread_block(npairs * 32 / na.rows, tblock);
         grid = 0;
     } else {
@@ -149,9 +152,11 @@ static cudaError_t newton_tile(const FindArgs& a, NewtonArgs na, int64_t npairs,
     }
     // two passes (and the mixed form's phases in launches of their own)
     // when the pairs fill the GPU several times over
-    const bool two = a.pstate && a.pause_list && (a.jst || !MIXED) && npairs >= kTwoPass;
+    const bool two = na.digits && a.pstate && a.pause_list && (a.jst || !MIXED) && npairs >= kTwoPass;
     na.first_pass = 0x7fffffff;
-    if (!two) {
+    if (!na.digits) {                                // no stored digits: one launch that makes them
+        err = launch_tile<n, KIND, true>(na, tab, launch, tblock, grid, s);
+    } else if (!two) {
         err = launch_tile<n, KIND>(na, tab, launch, tblock, grid, s);
     } else {
         na.pstate = a.pstate;

@@ -199,11 +199,18 @@ class Server:
         self.chunk_points = int(chunk_points)
         self.min_chunk = int(min_chunk)
         self.pairs_per_point = int(pairs_per_point)
-        self.resident = float(resident_bytes) + fg.fp_memory(handle)["resident"]
         self.budget = float(budget_bytes)
-        self.avail_total = self.budget - self.resident
-        if self.avail_total < self.bytes_for(min(self.min_chunk, self.chunk_points)):
-            raise ValueError("memory budget leaves no room for one chunk beside the resident state")
+        least = self.bytes_for(min(self.min_chunk, self.chunk_points))
+
+        def room():
+            self.resident = float(resident_bytes) + fg.fp_memory(handle)["resident"]
+            self.avail_total = self.budget - self.resident
+            return self.avail_total >= least
+        if not room():
+            # the mesh's stored node digits are what it can do without
+            fg.fp_set_node_digits(handle, False)
+            if not room():
+                raise ValueError("memory budget leaves no room for one chunk beside the resident state")
         self.streams = [torch.cuda.Stream(device=self.dev) for _ in range(max(1, int(streams)))]
         self.free_streams = list(self.streams)
         self.pool: Dict[int, List[_Buffers]] = collections.defaultdict(list)
