@@ -19,7 +19,8 @@ SOURCES = ["fp_host.cu", "fp_setup.cu", "fp_scan.cu", "fp_find.cu", "fp_find2.cu
            "fp_batch.cu", "fp_flux.cu", "fp_stream.cu", "fp_probe.cu", "fp_solve.cu", "fp_tile_mixed.cu"]
 HEADERS = ["fp_common.cuh", "fp_internal.h", "fp_handle.h", "fp_rank.cuh", "fp_newton.cuh", "fp_tile.cuh",
            "fp_tile_launch.cuh"]
-# sources compiled once per order n, with flags of their own
+# sources compiled once per order n, with flags of their own (the second's
+# orders are those of is_tile_order in fp_internal.h; a missing one does not link)
 PER_ORDER = {"fp_solve.cu": (range(2, 17), []), "fp_tile_mixed.cu": ([5, 7, 8, 9, 10], ["-fmad=false"])}
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 

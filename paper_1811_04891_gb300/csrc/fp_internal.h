@@ -47,10 +47,10 @@ cudaError_t scan_exclusive(const int32_t* in, int32_t* out, int64_t n, int32_t* 
 // Optional fused evaluation after classification, in the element-sorted pair
 // order: F fields, FP64 ([F][E][n3]) or double-float pairs; out [F][P].
 // threads per block of the Newton kernels when fp_opts.points_per_block is 0:
-// 64 for fp_find / fp_find_eval on hexahedra (measured 1 % faster than 128
-// for the FP64 form, the same for the mixed form, whose capped kernel takes
-// blocks of at most 128); 128 for quadrilaterals and for the workspace and
-// allocation-free calls, whose persistent grids are sized for it
+// 128, for which the tile kernels and the persistent grids are sized; 64 for
+// fp_find / fp_find_eval on hexahedra of the orders without tile kernels
+// (measured 1 % faster than 128 for the FP64 form, the same for the mixed
+// form)
 constexpr int kDefaultBlockFind3 = 64;
 constexpr int kDefaultBlock = 128;
 
@@ -135,15 +135,22 @@ struct FindArgs {
 //
 // The order decides alone, never the number of points, so that every entry
 // point gives a pair the same bits.  Lower orders have too little to contract,
-// higher ones more columns than a warp's accumulators hold.  FP64 form: faster
-// at every density for N = 3..9 (1.5 to 8 times).  Mixed form, fp_find in us,
-// one thread per pair / tiles, at 0.7, 5 and 600 points per element:
-//   N = 3  149/143  159/171   922/ 707     N = 4  183/159  193/190  1249/ 855
-//   N = 5  197/171  205/245  1438/1114     N = 6  249/198  274/280  1959/1318
-//   N = 7  281/183  315/276  2113/1289     N = 8  407/279  444/469  3178/2102
-//   N = 9  489/331  599/594  3617/2807
-// N = 3 and 5 lose 8 and 20 % at a few points per element (n^2 = 16 and 36
-// fill the k16 steps and n their columns badly) and keep one thread per pair.
+// higher ones more columns than a warp's accumulators hold.  fp_find in us, one
+// thread per pair / tiles, at 0.7, 5 and 600 (FP64, N >= 7: 300) points per
+// element:
+//   FP64 form    N = 3   681/ 287   830/ 323   9558/3046     N = 4  1079/ 316  1174/ 355  14314/3364
+//   N = 5  1561/ 372  1911/ 439  21040/4084     N = 6  2105/ 417  2684/ 516  29795/4601
+//   N = 7  3062/ 430  3473/ 523  21700/2633     N = 8  4584/ 530  6151/ 958  27972/3906
+//   N = 9  4892/ 606  6385/1085  35876/4293
+//   mixed form   N = 4   192/ 171   196/ 205   1258/ 873     N = 6   261/ 220   283/ 296   1960/1371
+//   N = 7   288/ 208   320/ 288   2105/1334     N = 8   407/ 310   453/ 497   3192/2181
+//   N = 9   478/ 361   640/ 635   3620/2868
+// Mixed form, N = 3 and 5: 8 and 20 % slower by tiles at a few points per
+// element (n^2 = 16 and 36 fill the k16 steps and n their columns badly): one
+// thread per pair.  On meshes whose digits exceed the L2 several times over
+// (17,576 elements, N = 7, mixed form) 1 to 10 points an element are slower by
+// tiles too (60,000 points 463/623, 400,000 1390/1143): a rule by the number
+// of points would give up the one above.
 constexpr bool is_tile_order(int n, bool mixed)
 {
     return mixed ? n == 5 || (n >= 7 && n <= 10) : n >= 4 && n <= 10;

@@ -1,6 +1,6 @@
 // fp_newton.cuh -- the box-constrained trust-region Newton solver of a
 // (point, candidate element) pair (Sec. 2.1) and its building blocks, shared
-// by the thread-per-pair kernels (fp_find.cu) and the tensor-core tile
+// by the thread-per-pair kernels (fp_solve.cu) and the tensor-core tile
 // kernels (fp_tile.cuh).
 #pragma once
 #include "fp_common.cuh"
@@ -479,14 +479,15 @@ struct NewtonArgs {
     int32_t ebase;
     int32_t* queue;             // work-queue counter (zeroed before the launch); null = grid-stride
     int tile;                   // sorted positions per work item (a multiple of 32)
-    double2* pstate;            // FP64 form: state of solves paused after the first pass's budget
-                                //   (rho, chord_fail + 4 flat + 8 it) per pair; null = one pass
+    double2* pstate;            // state of solves paused after the first pass's budget, per pair: rho and
+                                //   chord_fail + 4 it (k_newton) or + 4 flat + 8 it (tile kernels); null = one pass
     const unsigned char* digits;   // tile kernels: the elements' node digits (fp_tile.cuh)
     int rows;                   // tile kernels: sorted positions per warp, 1..32; 0: from the count on the device
     int32_t* pause_list;        // tile kernels: result positions of the solves paused after first_pass
     int32_t* pause_count;       //   evaluations (with pstate), capacity = all pairs; their number (zeroed before)
     bool resume;                // FP64 tile kernel: run the paused solves instead
     int list_blocks;            // mixed tile kernels, second launch: its first blocks run the listed solves
+    int list_spread;            //   a short list is spread over this many of them
     float* jst;                 // [9][cap] mixed tile kernels in two launches: the FP32 phase's Jacobian
     bool walk;                  // pair results (pres, prst, pstate) at sorted positions s (coalesced);
                                 //   otherwise at pair slots q.  Fallback lists hold the same index.

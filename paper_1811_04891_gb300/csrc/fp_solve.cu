@@ -404,6 +404,7 @@ static cudaError_t newton_form(const FindArgs& a, int64_t npairs, const BasisTab
     na.pause_count = nullptr;
     na.resume = false;
     na.list_blocks = 0;
+    na.list_spread = 0;
     na.jst = nullptr;
     na.rows = 32;
     cudaError_t err;

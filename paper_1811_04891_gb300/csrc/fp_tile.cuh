@@ -1376,7 +1376,8 @@ __device__ __forceinline__ void tile_final(const TileCtx<n, FLY>& X, const Newto
 enum { TILE_FP64 = 0, TILE_MIXED = 1, TILE_PHASE32 = 2, TILE_FINAL = 3 };
 
 // resident warps: the mixed kernels are capped at 128 registers (16 warps an
-// SM), the FP64 one at 168 (its shared memory allows 8 to 12 warps)
+// SM), the FP64 one at 168 (12 warps; at n = 9 and 10 its shared memory allows
+// 8 in blocks of 128 threads)
 template <int KIND>
 struct TileLB {
     static constexpr int threads = 128;
@@ -1519,13 +1520,11 @@ __device__ __forceinline__ void tile_rows_run(TileCtx<n, FLY>& X, const NewtonAr
 }
 
 // Listed rows lie in as many elements: a short list is spread over a wave of
-// blocks (the chain of a warp grows with its rows: 100,000 points in 4,096
-// elements, N = 7, 430 us; 490 with at least 16 rows a warp, 570 with 32), a
-// long one takes 32 rows a warp, whose FP64 steps cost the same for any number
-// (a batch of 24 problems 6,040 us with its lists spread over all list blocks,
-// 5,550 us so).
-constexpr int kListSpread = 152;
-
+// blocks (A.list_spread, one an SM: the chain of a warp grows with its rows;
+// 100,000 points in 4,096 elements, N = 7, 430 us; 490 with at least 16 rows a
+// warp, 570 with 32), a long one takes 32 rows a warp, whose FP64 steps cost
+// the same for any number (a batch of 24 problems 6,040 us with its lists
+// spread over all list blocks, 5,550 us so).
 // FLY: no stored digits (A.digits null); the launch's shared memory then ends
 // with the derivative table of the mixed form
 template <int n, int KIND, bool FLY = false>
@@ -1556,7 +1555,7 @@ __global__ void __launch_bounds__(TileLB<KIND>::threads, TileLB<KIND>::blocks) k
     };
     if (KIND == TILE_FINAL && (int)blockIdx.x < nl) {
         const PairRange L{0, (int64_t)*A.pause_count};
-        for_each_rows(A, L, rows_of(L.s1, min(nl, kListSpread), 0), false, (int)blockIdx.x, nl, [&](int64_t s0, int64_t s1) {
+        for_each_rows(A, L, rows_of(L.s1, min(nl, A.list_spread), 0), false, (int)blockIdx.x, nl, [&](int64_t s0, int64_t s1) {
             tile_rows_run<n, KIND, FLY>(X, A, tab, true, pl, fbl, fbc, s0, s1);
         });
         return;

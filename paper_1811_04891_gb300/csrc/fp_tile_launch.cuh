@@ -175,6 +175,7 @@ static cudaError_t newton_tile(const FindArgs& a, NewtonArgs na, int64_t npairs,
             // blocks for a list of one pair in twelve at 32 rows a warp (longer ones loop)
             na.first_pass = 0x7fffffff;
             na.list_blocks = (int)std::max<int64_t>(sm_count(), npairs / (12 * tblock));
+            na.list_spread = sm_count();
             if (err == cudaSuccess) err = launch_tile<n, TILE_FINAL>(na, tab, launch, tblock, grid, s);
         } else {
             err = launch_tile<n, TILE_FP64>(na, tab, launch, tblock, grid, s);
