@@ -79,6 +79,17 @@ TRAFFIC_PER_PAIR = {}
 HBM_FALLBACK_GBS = 6800.0
 
 
+def tile_fp64_ops(n: int) -> dict:
+    """Operations of the FP64 pipe that the FP64 form's tile kernel spends on a
+    row, n GLL points per direction: an evaluation with the Jacobian (three
+    bases with derivatives 39 n, their fixed-point halves 14 n, 9 n columns at
+    two operations, last contractions 12 n, step 60) and without it (15 n, 6 n,
+    6 n, 3 n, 40).  A located point takes at least two of each; the contraction
+    over n^3 nodes itself runs on the tensor cores."""
+    jac, val = 83 * n + 60, 30 * n + 40
+    return {"jac": jac, "value": val, "point": 2 * jac + 2 * val}
+
+
 def measured_hbm_gbs():
     """Measured copy bandwidth (GB/s) of the GB300s, else the
     fallback figure."""
@@ -287,9 +298,21 @@ def roofline_form(form, P, F, kernel_ms, ms_per_step, peaks, hbm_gbs, pairs, coo
     t_bytes = step_bytes / (hbm_gbs * 1e9)
     t_step = max(t_newton + t_eval, t_bytes)
     traffic = TRAFFIC_PER_PAIR.get(form)
+    if form == "fp64":
+        ops = tile_fp64_ops(8)["point"]
+        ms = 1e3 * P * ops / (p64 / 2)
+        executed = {"pipe": "FP64", "ops_per_point": ops, "ms": ms, "frac": ms / kernel_ms["newton"],
+                    "note": "FP64-pipe operations a located point cannot do without in k_newton_tile, at P64 / 2 "
+                            "operations a second"}
+    else:
+        executed = {"pipe": "issue", "frac": None,
+                    "note": "bound by instruction issue and one warp's chain (profiles/k_newton_tile_N7.md)"}
     fp64_view = P * (SEED + K_ORACLE * ITER + F * EVAL1) / p64
     return {"bound": "alu", "achieved": achieved / 1e12, "peak": peak / 1e12, "unit": unit,
-            "frac": t_newton / kn, "traffic": None if traffic is None else traffic * pairs,
+            "frac": t_newton / kn,
+            "frac_note": "against sum factorisation on the ALU pipes; the tile kernels contract on the tensor cores, so it "
+                         "may exceed 1 and is no utilisation (see executed)",
+            "executed": executed, "traffic": None if traffic is None else traffic * pairs,
             "kernel": "k_newton_tile<8> + k_newton64_full<8>" if form == "mixed" else "k_newton_tile<8>",
             "kernel_ms": kernel_ms["newton"], "units_per_launch": P, "work_unit": "located point (true element only)",
             "unit_work": w, "pairs_per_launch": pairs, "roofline_ms": 1e3 * t_newton,

@@ -43,16 +43,19 @@
 // digits the next one is fetched while the current one is multiplied.  The
 // FP64 form takes dx/dr and dx/ds from the same node digits with h_i' h_j and
 // h_i h_j' on the left: a third of the memory, set-up time and L2 traffic of
-// digits of the derivatives for two more left factors.  Tiles
-// of 128 pairs per tcgen05.mma would leave most rows empty (1 to 300 pairs
-// per element are typical), and the 16-row form is already bound by building
-// the digits, by the latency of its chain (16 warps an SM) and by issue
-// rather than by its 605 TFLOP/s (measured).
+// digits of the derivatives for two more left factors.  Tiles of 128 pairs
+// per tcgen05.mma would leave most rows empty (1 to 300 pairs per element are
+// typical), and the 16-row form is not bound by the tensor pipe (18 % busy in
+// the FP64 form's first pass, 30 % in the mixed form's two launches): the FP64
+// form is by the FP64 pipe (78 %: bases, columns, last contraction, 3x3
+// solves; 16 clocks of an SM a warp's operation), the mixed form by issue and
+// one warp's chain (46 % and 39 % of the issue slots with 13 and 14 of 16
+// warps).
 //
 // Measured (fp_find, N = 7, before = one thread per pair): 1.0e7 points in
-// 32,768 elements, mixed form, this stage 25.8 -> 14.9 ms; 3.0e5 points in
-// 1,000 elements, FP64 form, whole find 9.9 -> 2.5 ms; 1,501 points in 216
-// elements, N = 6, FP64 form, 1.95 -> 0.33 ms.
+// 32,768 elements, mixed form, this stage 25.8 -> 16.7 ms; 3.0e5 points in
+// 1,000 elements, FP64 form, whole find 21.7 -> 2.6 ms; 1,501 points in 216
+// elements, N = 6, FP64 form, 1.95 -> 0.43 ms.
 #pragma once
 #include <cuda_fp16.h>
 
@@ -1376,8 +1379,8 @@ __device__ __forceinline__ void tile_final(const TileCtx<n, FLY>& X, const Newto
 enum { TILE_FP64 = 0, TILE_MIXED = 1, TILE_PHASE32 = 2, TILE_FINAL = 3 };
 
 // resident warps: the mixed kernels are capped at 128 registers (16 warps an
-// SM), the FP64 one at 168 (12 warps; at n = 9 and 10 its shared memory allows
-// 8 in blocks of 128 threads)
+// SM), the FP64 one at 168 (12 warps); in blocks of 128 threads shared memory
+// leaves 12 and 8 at n = 9, 8 and 8 at n = 10
 template <int KIND>
 struct TileLB {
     static constexpr int threads = 128;
