@@ -73,9 +73,10 @@ def work_for_order(n: int) -> dict:
 WORK = {"fp64": {"f64": SEED + K_ORACLE * ITER, "f32": 0.0, "f64acc": 0.0},
         "mixed": {"f64": 0.0, "f32": SEED + K_ORACLE * ITER, "f64acc": FINAL}}
 # DRAM bytes (read + written) per (point, candidate element) pair of the Newton
-# stage, from a one-pass ncu capture of its launches at this full size; empty:
-# not captured for the tensor-core kernels.
-TRAFFIC_PER_PAIR = {}
+# stage, from one-pass ncu captures of its launches at this full size
+# (dram__bytes_read.sum + dram__bytes_write.sum of k_newton_tile's two launches
+# over 10.2 M pairs, find alone; profiles/k_newton_tile_N7.md).
+TRAFFIC_PER_PAIR = {"mixed": 1723.0, "fp64": 1317.0}
 HBM_FALLBACK_GBS = 6800.0
 
 
